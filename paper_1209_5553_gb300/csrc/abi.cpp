@@ -118,6 +118,8 @@ erem_status check_flags(erem_ctx* c) {
     return fail(c, EREM_ENONFINITE, "non-finite value in an input field or its derived coefficients");
   if (c->ctrl_h->flags & FLAG_BAD_INPUT)
     return fail(c, EREM_EINVAL, "negative conductivity, porosity outside [0,1] or non-positive capacity");
+  if (c->ctrl_h->flags & FLAG_TIMEOUT)
+    return fail(c, EREM_ETIMEOUT, "a wait of the resident Leja kernel ran out");
   return EREM_OK;
 }
 
@@ -471,9 +473,17 @@ erem_status leja_interp(erem_ctx* c, const double* u, const double* fused_T, int
   // taping (phi_1 of erem_step): the terms write q_m straight into the tape,
   // slot m of this interpolation, when the arena has room for every term
   const size_t qbytes = (size_t)c->Np * (c->prec == EREM_FP32_BULK ? sizeof(float) : sizeof(double));
+  // grids that fit on the chip: all the terms of the table in one resident
+  // launch (taped or not)
+  const bool res = o.avg_window <= 60 && leja_res_fits(c);
+  if (res && !c->res_msg) {
+    EREM_TRY(dalloc(c, &c->res_part, res_part_bytes(c)));
+    EREM_TRY(dalloc(c, &c->res_msg, res_msg_bytes(c)));
+  }
   char* slot0 = nullptr;
   if (c->rec_ok && phi == 1) {
-    const size_t need = (size_t)(forced ? forced : *M_avail) + 1;
+    // the resident form also keeps the vectors past the table's last term
+    const size_t need = (size_t)(forced ? forced : *M_avail + (res ? kResLag : 0)) + 1;
     if (c->tape_used + need * qbytes <= c->tape_cap) {
       slot0 = c->tape + c->tape_used;
       c->rec.q_off.push_back(c->tape_used);
@@ -485,19 +495,26 @@ erem_status leja_interp(erem_ctx* c, const double* u, const double* fused_T, int
   // small grids, untaped: each launch takes the stopping test of the term
   // before it (k_leja_term_lag), so the launch after the stopping term is
   // needed too: it completes P
-  const int lag = (c->term_lag && !slot0) ? 1 : 0;
+  // resident launches are lagged in the same way
+  const int lag = res ? kResLag : (c->term_lag && !slot0) ? 1 : 0;
   if (lag) c->last_lag = true;
   int m = 1, qin = 0;
-  int chunk = forced ? forced + lag : std::max(4, c->last_degree + 2 + lag);
+  int chunk = res ? kResTerms : forced ? forced + lag : std::max(4, c->last_degree + 2 + lag);
   // the terms [first, last] of every chunk of launches, in order; with
   // time_terms a pair of events brackets each chunk (not each launch: an
   // event between two terms would stop the next one from being scheduled
   // while the previous one ends)
   std::vector<std::pair<int, int>> chunks;
   while (true) {
-    const int end = forced ? forced + lag : std::min(*M_avail + lag, m + chunk - 1);
+    const int last = (forced ? forced : *M_avail) + lag;
+    const int end = std::min(last, m + chunk - 1);
     if (o.time_terms) cudaEventRecord(c->ev[2 * chunks.size()], s);
-    for (int mm = m; mm <= end; ++mm) {
+    if (res) {
+      EREM_CUDA(c, launch_leja_res(c, m, end, *M_avail + 1, forced && end == last ? 0 : 1,
+                                   slot0 ? (forced ? forced : end) : 0, slot0, qbytes, cg, s));
+      qin = end & 1;
+    }
+    for (int mm = m; !res && mm <= end; ++mm) {
       if (slot0)
         launch_leja_term_ptr(c, mm, slot0 + (size_t)(mm - 1) * qbytes, slot0 + (size_t)mm * qbytes,
                              cg, s);
@@ -518,9 +535,13 @@ erem_status leja_interp(erem_ctx* c, const double* u, const double* fused_T, int
       *nonfinite = *failed = true;
       return EREM_OK;
     }
-    if (forced) {
+    if (forced && end == last) {
       *degree = forced;
       break;
+    }
+    if (forced) {
+      m = end + 1;
+      continue;
     }
     if (h.done && !h.fail) {
       *degree = h.degree;
@@ -533,7 +554,7 @@ erem_status leja_interp(erem_ctx* c, const double* u, const double* fused_T, int
     if (end >= *M_avail + lag) {  // table exhausted below m_max: extend it
       *M_avail = mcap;
       EREM_TRY(prepare_dd(c, S, *M_avail, s, phi));
-      if (slot0 && c->tape_used + ((size_t)mcap + 1) * qbytes > c->tape_cap) {
+      if (slot0 && c->tape_used + ((size_t)mcap + 1 + lag) * qbytes > c->tape_cap) {
         // the tape cannot hold the longer interpolation: go on untaped (the
         // remaining terms continue from the last taped slot)
         EREM_CUDA(c, cudaMemcpyAsync(c->q[qin], slot0 + (size_t)(end)*qbytes, qbytes,
@@ -543,7 +564,7 @@ erem_status leja_interp(erem_ctx* c, const double* u, const double* fused_T, int
       }
     }
     m = end + 1;
-    chunk = 8;
+    if (!res) chunk = 8;
   }
   if (o.time_terms && tt) {
     // a chunk's time includes its launches after the stop (they return at
@@ -556,7 +577,7 @@ erem_status leja_interp(erem_ctx* c, const double* u, const double* fused_T, int
       if (cudaEventElapsedTime(&ms, c->ev[2 * j], c->ev[2 * j + 1]) == cudaSuccess) {
         tt->ms += ms;
         tt->terms += std::min(last, *degree) - first + 1;
-        tt->launches += last - first + 1;
+        tt->launches += res ? 1 : last - first + 1;
       }
     }
   }
@@ -1315,6 +1336,16 @@ erem_status erem_create(const erem_grid* grid, const erem_physics* phys, erem_pr
   }
   c->term_grid = std::min(c->red_blocks, term_waves * c->sm_count * leja_term_blocks_per_sm(c));
   if (const char* e = std::getenv("EREM_TERM_PDL")) c->pdl = std::atoi(e) != 0;  // tuning override
+  // the resident Leja kernel needs co-resident CTAs with most of an SM's
+  // shared memory; EREM_TERM_LAG (below) asks for launches term by term
+  int coop = 0;
+  if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&c->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device) !=
+          cudaSuccess) {
+    cudaGetLastError();
+    coop = 0;
+  }
+  c->res_ok = coop != 0 && !std::getenv("EREM_TERM_LAG");
   c->term_lag = Np <= kLagCells;
   if (const char* e = std::getenv("EREM_TERM_LAG")) c->term_lag = std::atoi(e) != 0;  // override
   const size_t np = (size_t)Np, nf = (size_t)g.ny * g.nz;
@@ -1406,6 +1437,8 @@ erem_status erem_destroy(erem_ctx* c) {
       if (p) cudaFree(p);
   if (c->kr_host) cudaFreeHost(c->kr_host);
   if (c->red_cnt) cudaFree(c->red_cnt);
+  if (c->res_msg) cudaFree(c->res_msg);
+  if (c->res_part) cudaFree(c->res_part);
   if (c->ctrl) cudaFree(c->ctrl);
   if (c->ctrl_h) cudaFreeHost(c->ctrl_h);
   if (c->dd_h) cudaFreeHost(c->dd_h);

@@ -22,8 +22,9 @@ constexpr int kMgCoarsest = 512;   // cells of the coarsest multigrid level, at 
 constexpr int kRedSlots = 4;       // reduction values per block
 constexpr double kRowSumNoDiag = 0x1p-28;  // largest relative interior row sum for a diagonal-free Leja copy
 
-// Bits of Ctrl::flags raised by the set-up kernels.
-enum : int { FLAG_NONFINITE = 1, FLAG_BAD_INPUT = 2 };
+// Bits of Ctrl::flags raised by the set-up kernels (and FLAG_TIMEOUT by a wait
+// of the resident Leja kernel that ran out).
+enum : int { FLAG_NONFINITE = 1, FLAG_BAD_INPUT = 2, FLAG_TIMEOUT = 4 };
 
 // Parameters of the Leja stopping test of one substep (§4.2).
 struct StopParams {
@@ -171,6 +172,7 @@ struct SmgLevel {
 constexpr int kDdShort = 48;    // divided differences of a level's first table
 constexpr int kDdThreads = 8;   // host threads of a divided-difference table
 constexpr long long kLagCells = 4500000;  // padded cells below which Leja terms run lagged
+constexpr int kResMinVecs = 32;   // vectors of a block of the resident Leja kernel, at least
 
 struct DDEntry {
   double c = 0, gamma = 0;
@@ -192,6 +194,14 @@ struct erem_ctx {
   bool pdl = true;        // Leja terms launched as programmatic dependents
   bool term_lag = false;  // small grids: each term's test taken by the next launch (k_leja_term_lag)
   mutable bool last_lag = false;  // the current call ran lagged terms
+  // resident Leja kernel (leja_resident.cu): messages and partial sums of its
+  // CTAs (allocated on first use), and the number its next launch counts from
+  bool res_ok = false;
+  int smem_optin = 0;             // shared memory a CTA may have
+  int res_hy = 0, res_hz = 0;     // rows of a CTA's block (0: not chosen yet)
+  void* res_msg = nullptr;
+  void* res_part = nullptr;
+  unsigned res_base = 1;
   std::string err;
 
   // stored fields (padded, FP64)
@@ -390,6 +400,15 @@ void launch_pfix(const erem_ctx* c, const void* q, int M, cudaStream_t s);
 // other blocks compute term m and add d_{m-1} q_{m-1} to P; m = 1 starts P
 // = d_0 p0.  The launch after the stopping term completes P.
 void launch_leja_term_lag(const erem_ctx* c, int m, int qin, double cg, cudaStream_t s);
+// Resident form (leja_resident.cu): terms m0 .. m1 in one cooperative launch,
+// where the grid's Leja working set fits on the chip.
+bool leja_res_fits(erem_ctx* c);
+constexpr int kResLag = 2;        // terms past the table's last one that complete P
+constexpr int kResTerms = 240;    // terms of one launch, at most
+size_t res_msg_bytes(const erem_ctx* c);
+size_t res_part_bytes(const erem_ctx* c);
+cudaError_t launch_leja_res(erem_ctx* c, int m0, int m1, int ndd, int keep_q, int tape_to, char* tape,
+                            size_t qbytes, double cg, cudaStream_t s);
 void launch_lincomb(const erem_ctx* c, double* out, double a, const double* x, double b,
                     const double* y, cudaStream_t s);
 

@@ -1047,9 +1047,15 @@ k_leja_term_lag(const Tq* __restrict__ qi, Tq* __restrict__ qo, double* __restri
       if constexpr (sizeof(Tq) == 4) sq = fmaf(a, a, sq);
       else acc = fma(a, a, acc);
     }
+    // a branch on m, not a choice between two results: either form costs one
+    // FP64 operation a cell, and the FP64 pipe is the scarce unit
+    if (m == 1) {
 #pragma unroll
-    for (int k = 0; k < VEC; ++k)
-      p[k] = m == 1 ? d0 * p[k] : fma(dprev, to_f64_fast(qc[k]), p[k]);
+      for (int k = 0; k < VEC; ++k) p[k] = d0 * p[k];
+    } else {
+#pragma unroll
+      for (int k = 0; k < VEC; ++k) p[k] = fma(dprev, to_f64_fast(qc[k]), p[k]);
+    }
     if constexpr (sizeof(Tq) == 4) {
       const float s = s_hi + sq;
       const float bp = s - s_hi;
