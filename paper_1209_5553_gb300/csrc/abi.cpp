@@ -813,14 +813,32 @@ erem_status run_forced(erem_ctx* c, double* out, const Opts& o, int m2_forced, e
                   std::to_string(o.max_doublings) + " substep doublings");
 }
 
+// What a step's front half forms of the right-hand side: nothing (the fused
+// first kernel does), ||T^n||_inf (the caller forms its own, or needs none), or
+// G(T^n) and ||T^n||_inf.
+enum RhsMode { RHS_NONE, RHS_NORM, RHS_FULL };
+
+erem_status launch_rhs_mode(erem_ctx* c, RhsMode mode, cudaStream_t s) {
+  if (mode == RHS_FULL) launch_rhs(c, c->Tn, c->vrhs, 1, s);
+  else if (mode == RHS_NORM) launch_yinf(c, c->Tn, s);
+  return EREM_OK;
+}
+
 // Assemble face fluxes (if fields changed or the fluid laws depend on T),
-// the cell form of J, G(T^n) and ||T^n||_inf; read alpha, beta back.
-erem_status assemble(erem_ctx* c, bool faces, bool rhs, cudaStream_t s) {
+// the cell form of J and what `rhs` asks for; read alpha, beta back.
+erem_status assemble(erem_ctx* c, bool faces, RhsMode rhs, cudaStream_t s) {
   if (faces) launch_faces(c, s);
   launch_cellJ(c, s);
-  if (rhs) launch_rhs(c, c->Tn, c->vrhs, 1, s);
+  EREM_TRY(launch_rhs_mode(c, rhs, s));
   EREM_TRY(check_launch(c, "assembly"));
   EREM_TRY(read_ctrl(c, s));
+  // G(T^n) that left the range of FP64 is an error also where nobody reads it:
+  // it can only with values of this size
+  if (rhs == RHS_NORM && !(c->ctrl_h->yinf < 1e100 && std::fabs(c->ctrl_h->gmin) < 1e100 &&
+                           std::fabs(c->phys.T_inflow) < 1e100)) {
+    launch_rhs(c, c->Tn, c->vrhs, 1, s);
+    EREM_TRY(read_ctrl(c, s));
+  }
   EREM_TRY(check_flags(c));
   // FP32-bulk: where every row of J off the inflow plane sums to zero (a
   // uniform temperature is transported nowhere; the discrete flux is
@@ -830,7 +848,7 @@ erem_status assemble(erem_ctx* c, bool faces, bool rhs, cudaStream_t s) {
   {
     const char* e = std::getenv("EREM_LEJA_DIAG");
     const bool keep_diag = e && std::atoi(e) != 0;
-    c->jl_nodiag = c->jl_r0 && !keep_diag && c->ctrl_h->rowsum <= kRowSumNoDiag;
+    c->jl_nodiag = c->jl_r0 && !keep_diag && c->ctrl_h->rowsum == 0.0;
   }
   set_interval(c);
   if (!std::isfinite(c->alpha) || !std::isfinite(c->beta))
@@ -875,7 +893,7 @@ erem_status rescale_jl(erem_ctx* c, cudaStream_t s) {
 // assembly when needed, G(T^n) into vrhs.  *Tdev receives T's device view.
 erem_status prepare_step(erem_ctx* c, double* T, const double* p, const double* lnk,
                          const double* phi, const double* lam, double dt, bool need_interval,
-                         cudaStream_t s, double** Tdev, bool fused = false) {
+                         cudaStream_t s, double** Tdev, bool fused = false, bool norm_only = false) {
   if (!T) return fail(c, EREM_EINVAL, "T is NULL");
   if (!(dt > 0.0) || !std::isfinite(dt)) return fail(c, EREM_EINVAL, "dt must be finite and > 0");
   const int nnull = (p == nullptr) + (lnk == nullptr) + (phi == nullptr) + (lam == nullptr);
@@ -888,9 +906,9 @@ erem_status prepare_step(erem_ctx* c, double* T, const double* p, const double* 
   EREM_TRY(resolve(c, 0, T, true, s, Tdev));
   const bool tdep = c->phys.fluid_model != 0;
   // the fused first kernel of run_phi1 computes G(T) and T^n itself
-  const bool rhs_here = !(fused && !tdep);
+  const RhsMode rhs_here = (fused && !tdep) ? RHS_NONE : norm_only ? RHS_NORM : RHS_FULL;
   const bool assemble_now = fields || tdep || !c->have_state;
-  if (rhs_here || assemble_now) launch_pack(c, *Tdev, c->Tn, s);
+  if (rhs_here != RHS_NONE || assemble_now) launch_pack(c, *Tdev, c->Tn, s);
   if (fields) EREM_TRY(load_fields(c, p, lnk, phi, lam, s));
   const double old_dt = c->dt;
   c->dt = dt;
@@ -899,7 +917,7 @@ erem_status prepare_step(erem_ctx* c, double* T, const double* p, const double* 
     c->jl_valid = false;
     c->have_state = true;
   } else {
-    if (rhs_here) launch_rhs(c, c->Tn, c->vrhs, 1, s);
+    EREM_TRY(launch_rhs_mode(c, rhs_here, s));
     EREM_TRY(check_launch(c, "rhs"));
     if (dt != old_dt) {
       set_interval(c);
@@ -1512,7 +1530,8 @@ erem_status erem_set_state(erem_ctx* c, const double* T, const double* p, const 
   double* Td;
   c->have_state = false;
   c->last_S = 1;  // a new run starts from one substep
-  EREM_TRY(prepare_step(c, const_cast<double*>(T), p, lnk, phi, lam, dt, true, s, &Td));
+  // (the steps form G(T^n) themselves, phi1_apply needs the norm only)
+  EREM_TRY(prepare_step(c, const_cast<double*>(T), p, lnk, phi, lam, dt, true, s, &Td, false, true));
   EREM_CUDA(c, cudaStreamSynchronize(s));
   return EREM_OK;
 }
@@ -1639,7 +1658,7 @@ erem_status erem_step_forced(erem_ctx* c, double* T, double dt, double T_in, dou
     EREM_TRY(dalloc_t(c, &c->fin_p2, (size_t)c->Np));
   }
   double* Td = nullptr;
-  EREM_TRY(prepare_step(c, T, p, lnk, phi, lam, dt, true, s, &Td, false));
+  EREM_TRY(prepare_step(c, T, p, lnk, phi, lam, dt, true, s, &Td, false, true));
   launch_inflow_forced(c, T_in, T_in_rate, c->fin_b, c->fin_w, s);
   launch_japply_add(c, c->Tn, c->fin_b, c->vrhs, s);  // G(T^n, t_n) = J T^n + b(T_in)
   EREM_TRY(check_launch(c, "forced right-hand side"));

@@ -63,7 +63,7 @@ struct Ctrl {
   double yinf;     // ||T^n||_inf of the current state
   double gmin, gmax;   // Gershgorin bounds of J (before the factor dt)
   double flux_in, vmax;
-  double rowsum;   // max over cells off the x = 0 plane of |row sum of J| / sum of |off-diagonals|
+  double rowsum;   // 1 if a row sum of J off the x = 0 plane is above kRowSumNoDiag sum |couplings|, else 0
   StopParams sp;
   double lin[K_NLIN];
   double e[kMaxTerms + 2];  // error estimates e_1 .. e_m of the substep
@@ -380,6 +380,7 @@ void launch_faces(const erem_ctx* c, cudaStream_t s);
 void launch_cellJ(const erem_ctx* c, cudaStream_t s);
 void launch_scale_jl(const erem_ctx* c, double sc, cudaStream_t s);
 void launch_rhs(const erem_ctx* c, const double* T, double* G, int set_yinf, cudaStream_t s);
+void launch_yinf(const erem_ctx* c, const double* T, cudaStream_t s);  // -> ctrl->yinf
 void launch_inflow_forced(const erem_ctx* c, double T_in, double rate, double* b, double* w,
                           cudaStream_t s);
 void launch_sumsq(const erem_ctx* c, const double* x, cudaStream_t s);  // -> ctrl->lin[K_EMB]

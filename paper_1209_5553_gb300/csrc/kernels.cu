@@ -34,7 +34,21 @@ __device__ __forceinline__ void cell_of(int i, const Geo& g, int& ix, int& iy, i
   ip = ix + g.px * r;
 }
 
-__device__ __forceinline__ bool finite(double x) { return isfinite(x); }
+// Comparisons on the bits of FP64 values: an FP64 compare takes a slot of the
+// FP64 pipe, which bounds the set-up kernels (two operations per clock and
+// SM), integer instructions do not.
+__device__ __forceinline__ bool finite(double x) { return bits_finite(abs_bits(x)); }
+// the sign bit: x < 0 for every x but -0.0 and NaN
+__device__ __forceinline__ bool neg(double x) { return __double2hiint(x) < 0; }
+// x's rank as an unsigned integer: a < b for doubles is rank(a) < rank(b)
+// (-0.0 below +0.0; NaNs outside the infinities)
+__device__ __forceinline__ unsigned long long rank_of(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  return (b >> 63) ? ~b : b | 0x8000000000000000ULL;
+}
+__device__ __forceinline__ double of_rank(unsigned long long r) {
+  return __longlong_as_double((long long)((r >> 63) ? r & 0x7fffffffffffffffULL : ~r));
+}
 
 // Fluid laws (fluid_model = 1): rho/rho0 = 1 - 3e-4 (T - 20),
 // mu/mu0 = exp(-0.02 (T - 20)); X = rho/rho0 * T and its T-derivative.
@@ -130,6 +144,7 @@ __global__ void k_lincomb(double* __restrict__ out, double a, const double* __re
 // ---------------------------------------------------------------------------
 struct FaceOut {
   double *Lx, *Ly, *Lz, *Fx, *Fy, *Fz, *icap, *LD0, *F0;
+  double* dX;  // dX/dT of every cell (T-dependent fluid), else null
 };
 struct FieldIn {
   const double *lnk, *phi, *lam, *p, *T;  // padded
@@ -147,9 +162,11 @@ __global__ void k_mobility(const double* __restrict__ lnk, const double* __restr
     int ix, iy, iz, ip;
     cell_of(i, g, ix, iy, iz, ip);
     const int j = in_padded ? ip : i;  // lnk and T in the padded or the caller's layout
-    const double Ti = T ? T[j] : 20.0;
-    const double mi = darcy ? exp(lnk[j]) / mu_rel(Ti, ph.fm)
-                            : exp(lnk[j]) * rho_rel(Ti, ph.fm) / mu_rel(Ti, ph.fm);
+    double mi = exp(lnk[j]);
+    if (ph.fm) {  // a linear fluid has density and viscosity 1: no FP64 division by it
+      const double Ti = T ? T[j] : 20.0;
+      mi = darcy ? mi / mu_rel(Ti, 1) : mi * rho_rel(Ti, 1) / mu_rel(Ti, 1);
+    }
     bad |= !finite(mi);
     m[ip] = mi;
   }
@@ -168,7 +185,7 @@ __global__ void k_faces(FieldIn in, const double* __restrict__ m, FaceOut o, Geo
     const double pi = in.p[ip];
     const double phi = in.phi[ip];
     bad |= !finite(mi) | !finite(li) | !finite(pi) | !finite(phi) | !finite(Ti);
-    inval |= (li < 0.0) | (phi < 0.0) | (phi > 1.0);
+    inval |= (neg(li) && li != 0.0) | (neg(phi) && phi != 0.0) | (rank_of(phi) > rank_of(1.0));
     // + x face
     if (ix < g.nx - 1) {
       const int j = ip + 1;
@@ -205,8 +222,9 @@ __global__ void k_faces(FieldIn in, const double* __restrict__ m, FaceOut o, Geo
       o.LD0[r] = ph.ax * li / (0.5 * ph.hx);
       o.F0[r] = ph.rhoc_f * (ph.ax * mi / (0.5 * ph.hx)) * (ph.head_left - pi);
     }
+    if (o.dX) o.dX[ip] = dXof(Ti, 1);
     const double C = phi * ph.rhoc_f + (1.0 - phi) * ph.rhoc_s;
-    inval |= !(C > 0.0);
+    inval |= neg(C) | (abs_bits(C) == 0ULL) | (abs_bits(C) > 0x7ff0000000000000ULL);  // !(C > 0)
     o.icap[ip] = 1.0 / (C * ph.vol);
   }
   if (bad) atomicOr(flags, FLAG_NONFINITE);
@@ -226,79 +244,72 @@ struct JOut {
   double* b0;    // constant part of G at the x = 0 cells (linear fluid model)
 };
 
-__global__ void k_cellJ(FaceIn f, const double* __restrict__ T, JOut o, Geo g, Phys ph,
+// FM is the fluid model.  FP64 operations bound this kernel (39 per cell in 3D
+// with the linear fluid; 88 when the upwind choices, extremes and checks were
+// FP64 compares and the row-sum test an FP64 division): 192^3 1070 -> 520 us.
+// dX (FM = 1): dX/dT of every cell, written by k_faces.
+template <int FM>
+__global__ void k_cellJ(FaceIn f, const double* __restrict__ dX, JOut o, Geo g, Phys ph,
                         double* part, unsigned* cnt, Ctrl* ctrl) {
   __shared__ double sh[NT / 32];
-  double gmin = INFINITY, gmax = -INFINITY, rmax = 0.0;
-  int bad = 0;
-  const int fm = ph.fm;
+  unsigned long long gmin = rank_of(INFINITY), gmax = rank_of(-INFINITY);
+  int bad = 0, tilted = 0;
   for (int i = blockIdx.x * NT + threadIdx.x; i < g.N; i += gridDim.x * NT) {
     int ix, iy, iz, ip;
     cell_of(i, g, ix, iy, iz, ip);
-    const double dXi = dXof(T[ip], fm);
+    const double dXi = FM ? dX[ip] : 1.0;
     double D = 0.0, W = 0.0, E = 0.0, S = 0.0, Nn = 0.0, B = 0.0, Tt = 0.0;
-    // + x face
-    {
-      const double F = f.Fx[ip];
-      if (ix < g.nx - 1) {
-        D -= f.Lx[ip] + (F >= 0.0 ? F * dXi : 0.0);
-        E = f.Lx[ip] + (F < 0.0 ? -F * dXof(T[ip + 1], fm) : 0.0);
-      } else {
-        D -= F * dXi;  // outflow face carries X_i for either sign
-      }
-    }
-    // - x face
+    // F > 0 leaves through a + face carrying X_i, F < 0 enters carrying X_j;
+    // every product and sum is rounded on its own
+    auto times = [](double F, double d) { return FM ? __dmul_rn(F, d) : F; };
+    auto plus = [&](int q, double L, double F, double& c) {
+      const bool in = neg(F);
+      D = __dsub_rn(D, __dadd_rn(L, in ? 0.0 : times(F, dXi)));
+      c = __dadd_rn(L, in ? times(-F, FM ? dX[q] : 1.0) : 0.0);
+    };
+    auto minus = [&](int q, double L, double F, double& c) {
+      const bool out = neg(F);
+      D = __dsub_rn(D, __dadd_rn(L, out ? times(-F, dXi) : 0.0));
+      c = __dadd_rn(L, out ? 0.0 : times(F, FM ? dX[q] : 1.0));
+    };
+    if (ix < g.nx - 1) plus(ip + 1, f.Lx[ip], f.Fx[ip], E);
+    else D = __dsub_rn(D, times(f.Fx[ip], dXi));  // outflow face carries X_i for either sign
     if (ix > 0) {
-      const double F = f.Fx[ip - 1];
-      D -= f.Lx[ip - 1] + (F < 0.0 ? -F * dXi : 0.0);
-      W = f.Lx[ip - 1] + (F >= 0.0 ? F * dXof(T[ip - 1], fm) : 0.0);
+      minus(ip - 1, f.Lx[ip - 1], f.Fx[ip - 1], W);
     } else {
       const int r = iy + g.ny * iz;
       const double F = f.F0[r];
       D -= f.LD0[r] + (F > 0.0 ? 0.0 : -F * dXi);
       if (o.b0)
-        o.b0[r] = f.icap[ip] * (f.LD0[r] * ph.T_in + (F > 0.0 ? F * Xof(ph.T_in, fm) : 0.0));
+        o.b0[r] = f.icap[ip] * (f.LD0[r] * ph.T_in + (F > 0.0 ? F * Xof(ph.T_in, FM) : 0.0));
     }
-    // +- y faces
-    if (iy < g.ny - 1) {
-      const double F = f.Fy[ip];
-      D -= f.Ly[ip] + (F >= 0.0 ? F * dXi : 0.0);
-      Nn = f.Ly[ip] + (F < 0.0 ? -F * dXof(T[ip + g.px], fm) : 0.0);
-    }
-    if (iy > 0) {
-      const double F = f.Fy[ip - g.px];
-      D -= f.Ly[ip - g.px] + (F < 0.0 ? -F * dXi : 0.0);
-      S = f.Ly[ip - g.px] + (F >= 0.0 ? F * dXof(T[ip - g.px], fm) : 0.0);
-    }
+    if (iy < g.ny - 1) plus(ip + g.px, f.Ly[ip], f.Fy[ip], Nn);
+    if (iy > 0) minus(ip - g.px, f.Ly[ip - g.px], f.Fy[ip - g.px], S);
     if (g.dim == 3) {
-      if (iz < g.nz - 1) {
-        const double F = f.Fz[ip];
-        D -= f.Lz[ip] + (F >= 0.0 ? F * dXi : 0.0);
-        Tt = f.Lz[ip] + (F < 0.0 ? -F * dXof(T[ip + g.plane], fm) : 0.0);
-      }
-      if (iz > 0) {
-        const double F = f.Fz[ip - g.plane];
-        D -= f.Lz[ip - g.plane] + (F < 0.0 ? -F * dXi : 0.0);
-        B = f.Lz[ip - g.plane] + (F >= 0.0 ? F * dXof(T[ip - g.plane], fm) : 0.0);
-      }
+      if (iz < g.nz - 1) plus(ip + g.plane, f.Lz[ip], f.Fz[ip], Tt);
+      if (iz > 0) minus(ip - g.plane, f.Lz[ip - g.plane], f.Fz[ip - g.plane], B);
     }
     const double ic = f.icap[ip];
-    D *= ic; W *= ic; E *= ic; S *= ic; Nn *= ic; B *= ic; Tt *= ic;
+    D *= ic; W *= ic; E *= ic; S *= ic; Nn *= ic;
     o.c[0][ip] = D; o.c[1][ip] = W; o.c[2][ip] = E; o.c[3][ip] = S; o.c[4][ip] = Nn;
-    if (g.dim == 3) { o.c[5][ip] = B; o.c[6][ip] = Tt; }
-    const double R = fabs(W) + fabs(E) + fabs(S) + fabs(Nn) + fabs(B) + fabs(Tt);
-    bad |= !finite(D) | !finite(R);
-    gmin = fmin(gmin, D - R);
-    gmax = fmax(gmax, D + R);
-    if (ix > 0) {  // the row sum relative to the couplings, off the Dirichlet inflow plane
-      const double rs = fabs(D + W + E + S + Nn + B + Tt);
-      rmax = fmax(rmax, R > 0.0 ? rs / R : (rs > 0.0 ? INFINITY : 0.0));
+    double R = fabs(W) + fabs(E) + fabs(S) + fabs(Nn);
+    double rs = D + W + E + S + Nn;
+    if (g.dim == 3) {
+      B *= ic; Tt *= ic;
+      o.c[5][ip] = B; o.c[6][ip] = Tt;
+      R = R + fabs(B) + fabs(Tt);
+      rs = rs + B + Tt;
     }
+    bad |= !finite(D) | !finite(R);
+    gmin = min(gmin, rank_of(D - R));
+    gmax = max(gmax, rank_of(D + R));
+    // the row sum relative to the couplings, off the Dirichlet inflow plane
+    if (ix > 0) tilted |= abs_bits(rs) > abs_bits(kRowSumNoDiag * R);
   }
   if (bad) atomicOr(&ctrl->flags, FLAG_NONFINITE);
-  const double bmin = block_reduce<1>(gmin, sh);
-  const double bmax = block_reduce<2>(gmax, sh);
-  const double brs = block_reduce<2>(rmax, sh);
+  const double bmin = block_reduce<1>(of_rank(gmin), sh);
+  const double bmax = block_reduce<2>(of_rank(gmax), sh);
+  const double brs = block_reduce<2>(tilted ? 1.0 : 0.0, sh);
   double vals[3] = {bmin, bmax, brs};
   if (publish_partials(part, cnt, vals, 3)) {
     const double a = gather_partials<1>(part, 0, sh);
@@ -317,21 +328,25 @@ __global__ void k_cellJ(FaceIn f, const double* __restrict__ T, JOut o, Geo g, P
 // interleaved layout of LejaCoef (tile of T cells).  skip = 1: the couplings
 // only (the diagonal is implied by the row sums, zero off the x = 0 plane),
 // and r0[row] = (Tq)(sc * row sum) at the x = 0 cells.
-template <typename Tq, int T>
-__global__ void k_scale_jl(JOut jc, Tq* __restrict__ out, double sc, int Np, int nc,
-                           float2* __restrict__ rsum, int skip, Tq* __restrict__ r0, int px) {
-  const int nout = nc - skip;
+template <typename Tq, int T, int NC, int SKIP>
+__global__ void k_scale_jl(JOut jc, Tq* __restrict__ out, double sc, int Np,
+                           float2* __restrict__ rsum, Tq* __restrict__ r0, int px) {
+  constexpr int NOUT = NC - SKIP;
   for (int i = blockIdx.x * NT + threadIdx.x; i < Np; i += gridDim.x * NT) {
-    const size_t base = (size_t)(i / T) * nout * T + (i % T);
-    for (int k = skip; k < nc; ++k) out[base + (size_t)(k - skip) * T] = (Tq)(sc * jc.c[k][i]);
-    if (rsum || skip) {
+    const size_t base = (size_t)(i / T) * NOUT * T + (i % T);
+#pragma unroll
+    for (int k = SKIP; k < NC; ++k) out[base + (size_t)(k - SKIP) * T] = (Tq)(sc * jc.c[k][i]);
+    // row sums: of every cell (rsum), or of the x = 0 cells only, where the
+    // diagonal-free kernels read them
+    if (SKIP ? i % px == 0 : rsum != nullptr) {
       double r = 0.0;  // row sum r_i of J (FP64)
-      for (int k = 0; k < nc; ++k) r += jc.c[k][i];
+#pragma unroll
+      for (int k = 0; k < NC; ++k) r += jc.c[k][i];
       if (rsum) {  // as a float pair hi + lo
         const float hi = (float)r;
         rsum[i] = make_float2(hi, (float)(r - (double)hi));
       }
-      if (skip && i % px == 0) r0[i / px] = (Tq)(sc * r);
+      if (SKIP) r0[i / px] = (Tq)(sc * r);
     }
   }
 }
@@ -400,6 +415,28 @@ __global__ void k_rhs(FaceIn f, const double* __restrict__ T, double* __restrict
   if (bad) atomicOr(&ctrl->flags, FLAG_NONFINITE);
   if (!set_yinf) return;
   const double bmax = block_reduce<2>(tmax, sh);
+  double vals[1] = {bmax};
+  if (publish_partials(part, cnt, vals, 1)) {
+    const double a = gather_partials<2>(part, 0, sh);
+    if (threadIdx.x == 0) {
+      ctrl->yinf = a;
+      *cnt = 0;
+    }
+  }
+}
+
+// ||T||_inf alone, for callers that form their right-hand side elsewhere (pads
+// hold 0)
+__global__ void k_yinf(const double* __restrict__ T, int Np, double* part, unsigned* cnt, Ctrl* ctrl) {
+  __shared__ double sh[NT / 32];
+  unsigned long long tmax = 0ULL;
+  for (int v = blockIdx.x * NT + threadIdx.x; v < Np / 4; v += gridDim.x * NT) {
+    const double2 a = *reinterpret_cast<const double2*>(T + 4 * v);
+    const double2 b = *reinterpret_cast<const double2*>(T + 4 * v + 2);
+    tmax = max(max(tmax, max(abs_bits(a.x), abs_bits(a.y))), max(abs_bits(b.x), abs_bits(b.y)));
+  }
+  if (!bits_finite(tmax)) atomicOr(&ctrl->flags, FLAG_NONFINITE);
+  const double bmax = block_reduce<2>(__longlong_as_double((long long)tmax), sh);
   double vals[1] = {bmax};
   if (publish_partials(part, cnt, vals, 1)) {
     const double a = gather_partials<2>(part, 0, sh);
@@ -1625,14 +1662,15 @@ struct PresArr {
   double *x, *r, *z, *d0, *d1, *Ad, *Ux, *Uy, *Uz, *diag, *b;
 };
 
-// TPFA pressure matrix from the cell mobilities m: upper couplings, diagonal
-// (with the Dirichlet faces at x = 0 and x = 1) and right-hand side
+// TPFA pressure matrix from the cell mobilities m: the couplings to the next
+// cell in x, y and z.  The diagonal sums them in a pass of its own
+// (k_pres_diag): formed here it would evaluate every harmonic mean twice, and
+// their FP64 divisions bound the pass (128^3: 374 us, now 151 + 59)
 __global__ void k_pres_faces(const double* __restrict__ m, PresArr a, Geo g, Phys ph) {
   for (int i = blockIdx.x * NT + threadIdx.x; i < g.N; i += gridDim.x * NT) {
     int ix, iy, iz, ip;
     cell_of(i, g, ix, iy, iz, ip);
     const double mi = m[ip];
-    double dg = 0.0, bb = 0.0;
     double ux = 0.0, uy = 0.0, uz = 0.0;
     if (ix < g.nx - 1) ux = harm(ph.ax, 0.5 * ph.hx, mi, m[ip + 1]);
     if (iy < g.ny - 1) uy = harm(ph.ay, 0.5 * ph.hy, mi, m[ip + g.px]);
@@ -1640,13 +1678,25 @@ __global__ void k_pres_faces(const double* __restrict__ m, PresArr a, Geo g, Phy
     a.Ux[ip] = ux;
     a.Uy[ip] = uy;
     if (g.dim == 3) a.Uz[ip] = uz;
-    dg += ux + uy + uz;
-    if (ix > 0) dg += harm(ph.ax, 0.5 * ph.hx, m[ip - 1], mi);
-    if (iy > 0) dg += harm(ph.ay, 0.5 * ph.hy, m[ip - g.px], mi);
-    if (g.dim == 3 && iz > 0) dg += harm(ph.az, 0.5 * ph.hz, m[ip - g.plane], mi);
-    const double uD = ph.ax * mi / (0.5 * ph.hx);
-    if (ix == 0) { dg += uD; bb += uD * ph.head_left; }
-    if (ix == g.nx - 1) { dg += uD; bb += uD * ph.head_right; }
+  }
+}
+
+// The diagonal (the six couplings of a cell and the Dirichlet faces at x = 0
+// and x = 1) and the right-hand side.
+__global__ void k_pres_diag(const double* __restrict__ m, PresArr a, Geo g, Phys ph) {
+  for (int i = blockIdx.x * NT + threadIdx.x; i < g.N; i += gridDim.x * NT) {
+    int ix, iy, iz, ip;
+    cell_of(i, g, ix, iy, iz, ip);
+    double dg = 0.0, bb = 0.0;
+    dg += a.Ux[ip] + a.Uy[ip] + (g.dim == 3 ? a.Uz[ip] : 0.0);
+    if (ix > 0) dg += a.Ux[ip - 1];
+    if (iy > 0) dg += a.Uy[ip - g.px];
+    if (g.dim == 3 && iz > 0) dg += a.Uz[ip - g.plane];
+    if (ix == 0 || ix == g.nx - 1) {
+      const double uD = ph.ax * m[ip] / (0.5 * ph.hx);
+      if (ix == 0) { dg += uD; bb += uD * ph.head_left; }
+      if (ix == g.nx - 1) { dg += uD; bb += uD * ph.head_right; }
+    }
     a.diag[ip] = dg;
     a.b[ip] = bb;
   }
@@ -1666,7 +1716,9 @@ __device__ __forceinline__ double pres_apply(const PresArr& a, const double* __r
   return v;
 }
 
-// r = b - A x, z = r / diag, d_old = 0; rz, rr, bb
+// r = b - A x, d_old = 0; rr, bb; with JAC also z = r / diag and rz (the other
+// preconditioners form their own, and skip the FP64 division)
+template <int JAC>
 __global__ void k_cg_init(PresArr a, Geo g, double tol, double* part, unsigned* cnt, Ctrl* ctrl) {
   __shared__ double sh[NT / 32];
   double rz = 0.0, rr = 0.0, bb = 0.0;
@@ -1674,11 +1726,13 @@ __global__ void k_cg_init(PresArr a, Geo g, double tol, double* part, unsigned* 
     int ix, iy, iz, ip;
     cell_of(i, g, ix, iy, iz, ip);
     const double r = a.b[ip] - pres_apply(a, a.x, ip, ix, iy, iz, g);
-    const double z = r / a.diag[ip];
     a.r[ip] = r;
-    a.z[ip] = z;
     a.d0[ip] = 0.0;
-    rz += r * z;
+    if (JAC) {
+      const double z = r / a.diag[ip];
+      a.z[ip] = z;
+      rz += r * z;
+    }
     rr += r * r;
     bb += a.b[ip] * a.b[ip];
   }
@@ -1704,31 +1758,60 @@ __global__ void k_cg_init(PresArr a, Geo g, double tol, double* part, unsigned* 
   }
 }
 
-// d_new = z + beta d_old; Ad = A d_new; (d, Ad) -> alpha.  z is the
-// preconditioned residual: FP64 (Jacobi) or FP32 (polynomial preconditioner).
+// d_new = z + beta d_old, four cells of the padded layout per thread.  z is
+// the preconditioned residual: FP64 (Jacobi) or FP32 (polynomial or multigrid
+// preconditioner).  A pass of its own: formed where the stencil needs it, it
+// would be computed seven times per cell (two FP64 operations each, and the
+// FP64 pipe bounds the stencil pass).
 template <typename Tz>
-__global__ void k_cg_dir(PresArr a, const Tz* __restrict__ z, const double* __restrict__ dold,
-                         double* __restrict__ dnew, Geo g, double* part, unsigned* cnt,
+__global__ void k_cg_newdir(const Tz* __restrict__ z, const double* __restrict__ dold,
+                            double* __restrict__ dnew, int Np, const Ctrl* ctrl) {
+  if (*(volatile const int*)&ctrl->lin_done) return;
+  const double beta = ctrl->lin[K_BETA];
+  for (int v = blockIdx.x * NT + threadIdx.x; v < Np / 4; v += gridDim.x * NT) {
+    double d[4], zz[4];
+    const double2 a = *reinterpret_cast<const double2*>(dold + 4 * v);
+    const double2 b = *reinterpret_cast<const double2*>(dold + 4 * v + 2);
+    if constexpr (sizeof(Tz) == 4) {
+      float zf[4];
+      ldv<float, 4>(zf, z + 4 * v);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) zz[j] = f2d_fast(zf[j]);
+    } else {
+      const double2 p = *reinterpret_cast<const double2*>(z + 4 * v);
+      const double2 q = *reinterpret_cast<const double2*>(z + 4 * v + 2);
+      zz[0] = p.x; zz[1] = p.y; zz[2] = q.x; zz[3] = q.y;
+    }
+    d[0] = fma(beta, a.x, zz[0]);
+    d[1] = fma(beta, a.y, zz[1]);
+    d[2] = fma(beta, b.x, zz[2]);
+    d[3] = fma(beta, b.y, zz[3]);
+    *reinterpret_cast<double2*>(dnew + 4 * v) = make_double2(d[0], d[1]);
+    *reinterpret_cast<double2*>(dnew + 4 * v + 2) = make_double2(d[2], d[3]);
+  }
+}
+
+// Ad = A d; (d, Ad) -> alpha.  With k_cg_newdir at 128^3: 10 + 41 us where
+// forming d inside took 91, at 1024^2 6 + 21 instead of 40 (FP64 operations
+// per cell in 3D: 1 + 8 instead of 23).
+__global__ void k_cg_dir(PresArr a, const double* __restrict__ d, Geo g, double* part, unsigned* cnt,
                          Ctrl* ctrl) {
   __shared__ double sh[NT / 32];
   if (*(volatile int*)&ctrl->lin_done) return;
-  const double beta = ctrl->lin[K_BETA];
   double dad = 0.0;
   for (int i = blockIdx.x * NT + threadIdx.x; i < g.N; i += gridDim.x * NT) {
     int ix, iy, iz, ip;
     cell_of(i, g, ix, iy, iz, ip);
-    auto dn = [&](int j) { return (double)z[j] + beta * dold[j]; };
-    const double di = dn(ip);
+    const double di = d[ip];
     double v = a.diag[ip] * di;
-    if (ix < g.nx - 1) v -= a.Ux[ip] * dn(ip + 1);
-    if (ix > 0) v -= a.Ux[ip - 1] * dn(ip - 1);
-    if (iy < g.ny - 1) v -= a.Uy[ip] * dn(ip + g.px);
-    if (iy > 0) v -= a.Uy[ip - g.px] * dn(ip - g.px);
+    if (ix < g.nx - 1) v -= a.Ux[ip] * d[ip + 1];
+    if (ix > 0) v -= a.Ux[ip - 1] * d[ip - 1];
+    if (iy < g.ny - 1) v -= a.Uy[ip] * d[ip + g.px];
+    if (iy > 0) v -= a.Uy[ip - g.px] * d[ip - g.px];
     if (g.dim == 3) {
-      if (iz < g.nz - 1) v -= a.Uz[ip] * dn(ip + g.plane);
-      if (iz > 0) v -= a.Uz[ip - g.plane] * dn(ip - g.plane);
+      if (iz < g.nz - 1) v -= a.Uz[ip] * d[ip + g.plane];
+      if (iz > 0) v -= a.Uz[ip - g.plane] * d[ip - g.plane];
     }
-    dnew[ip] = di;
     a.Ad[ip] = v;
     dad += di * v;
   }
@@ -1895,8 +1978,9 @@ __global__ void k_pc_sweep(PresArr a, PcArr p, const float* __restrict__ zprev,
 #pragma unroll
       for (int j = 0; j < 4; ++j)
         if (R.ix0 + j < g.nx) {
-          rz += (double)zn[j] * rr[j];
-          zad += (double)zn[j] * dd[j];
+          const double z = f2d_fast(zn[j]);  // integer instructions: the FP64 pipe keeps the two sums
+          rz += z * rr[j];
+          zad += z * dd[j];
         }
     }
   }
@@ -2273,37 +2357,46 @@ __global__ void k_sumsq(const double* __restrict__ x, Geo g, double* part, unsig
   }
 }
 
-// net Darcy inflow through x = 0 and the largest face speed |v| / |sigma|
-__global__ void k_pres_post(const double* __restrict__ m, const double* __restrict__ x, Geo g,
-                            Phys ph, double* part, unsigned* cnt, Ctrl* ctrl) {
+// Net Darcy inflow through x = 0 and the largest face speed |v| / |sigma|.
+// FM = 1: the harmonic means of the Darcy mobilities m = K / mu (padded).  FM
+// = 0: density and viscosity are 1, the means are the pressure couplings
+// themselves, and m is ln K in the caller's layout, read at the x = 0 and x =
+// 1 cells only.  |v| is compared per axis and divided by the face area once
+// per thread (a division per face bounded the pass: 128^3 327 -> 60 us).
+template <int FM>
+__global__ void k_pres_post(const double* __restrict__ m, PresArr a, Geo g, Phys ph, double* part,
+                            unsigned* cnt, Ctrl* ctrl) {
   __shared__ double sh[NT / 32];
-  double fin = 0.0, vmax = 0.0;
+  const double* __restrict__ x = a.x;
+  double fin = 0.0;
+  unsigned long long vx = 0ULL, vy = 0ULL, vz = 0ULL;
+  auto top = [](unsigned long long w, double v) {  // NaNs do not count
+    const unsigned long long b = abs_bits(v);
+    return b > w && b <= 0x7ff0000000000000ULL ? b : w;
+  };
   for (int i = blockIdx.x * NT + threadIdx.x; i < g.N; i += gridDim.x * NT) {
     int ix, iy, iz, ip;
     cell_of(i, g, ix, iy, iz, ip);
-    const double mi = m[ip];
     const double pi = x[ip];
+    const double mi = FM ? m[ip] : (ix == 0 || ix == g.nx - 1 ? exp(m[i]) : 0.0);
     if (ix == 0) {
       const double v = (ph.ax * mi / (0.5 * ph.hx)) * (ph.head_left - pi);
       fin += v;
-      vmax = fmax(vmax, fabs(v) / ph.ax);
+      vx = top(vx, v);
     }
-    if (ix < g.nx - 1) {
-      const double v = harm(ph.ax, 0.5 * ph.hx, mi, m[ip + 1]) * (pi - x[ip + 1]);
-      vmax = fmax(vmax, fabs(v) / ph.ax);
-    } else {
-      const double v = (ph.ax * mi / (0.5 * ph.hx)) * (pi - ph.head_right);
-      vmax = fmax(vmax, fabs(v) / ph.ax);
-    }
-    if (iy < g.ny - 1) {
-      const double v = harm(ph.ay, 0.5 * ph.hy, mi, m[ip + g.px]) * (pi - x[ip + g.px]);
-      vmax = fmax(vmax, fabs(v) / ph.ay);
-    }
-    if (g.dim == 3 && iz < g.nz - 1) {
-      const double v = harm(ph.az, 0.5 * ph.hz, mi, m[ip + g.plane]) * (pi - x[ip + g.plane]);
-      vmax = fmax(vmax, fabs(v) / ph.az);
-    }
+    if (ix < g.nx - 1)
+      vx = top(vx, (FM ? harm(ph.ax, 0.5 * ph.hx, mi, m[ip + 1]) : a.Ux[ip]) * (pi - x[ip + 1]));
+    else
+      vx = top(vx, (ph.ax * mi / (0.5 * ph.hx)) * (pi - ph.head_right));
+    if (iy < g.ny - 1)
+      vy = top(vy, (FM ? harm(ph.ay, 0.5 * ph.hy, mi, m[ip + g.px]) : a.Uy[ip]) * (pi - x[ip + g.px]));
+    if (g.dim == 3 && iz < g.nz - 1)
+      vz = top(vz, (FM ? harm(ph.az, 0.5 * ph.hz, mi, m[ip + g.plane]) : a.Uz[ip]) *
+                       (pi - x[ip + g.plane]));
   }
+  double vmax = __longlong_as_double((long long)vx) / ph.ax;
+  vmax = fmax(vmax, __longlong_as_double((long long)vy) / ph.ay);
+  if (g.dim == 3) vmax = fmax(vmax, __longlong_as_double((long long)vz) / ph.az);
   double vals[2] = {block_reduce<0>(fin, sh), 0.0};
   vals[1] = block_reduce<2>(vmax, sh);
   if (publish_partials(part, cnt, vals, 2)) {
@@ -2837,10 +2930,12 @@ void launch_finish(const erem_ctx* c, double* out, const double* base, const dou
 }
 
 // the cell mobilities K / mu(T) go to P (the Leja sum, which every step
-// initialises after the assembly); T is T^n, or u when visc_u is set
+// initialises after the assembly), dX/dT to w (written before it is read by
+// every step); T is T^n, or u when visc_u is set
 void launch_faces(const erem_ctx* c, cudaStream_t s) {
   FieldIn in{c->lnk, c->phi, c->lam, c->p, c->Tn};
-  FaceOut o{c->Lx, c->Ly, c->Lz, c->Fx, c->Fy, c->Fz, c->icap, c->LD0, c->F0};
+  FaceOut o{c->Lx, c->Ly, c->Lz, c->Fx, c->Fy, c->Fz, c->icap, c->LD0, c->F0,
+            c->phys.fluid_model ? c->w : nullptr};
   c->launches += 2;
   k_mobility<<<blocks_cells(c), NT, 0, s>>>(c->lnk, c->visc_u ? c->u : c->Tn, c->P, geo_of(c),
                                             phys_of(c), 1, 1, &c->ctrl->flags);
@@ -2852,8 +2947,12 @@ void launch_cellJ(const erem_ctx* c, cudaStream_t s) {
   for (int k = 0; k < 7; ++k) o.c[k] = c->jc[k];
   o.b0 = c->b0;
   ++c->launches;
-  k_cellJ<<<blocks_cells(c), NT, 0, s>>>(face_in(c), c->Tn, o, geo_of(c), phys_of(c), c->red_part,
-                                         c->red_cnt, c->ctrl);
+  if (c->phys.fluid_model)
+    k_cellJ<1><<<blocks_cells(c), NT, 0, s>>>(face_in(c), c->w, o, geo_of(c), phys_of(c), c->red_part,
+                                              c->red_cnt, c->ctrl);
+  else
+    k_cellJ<0><<<blocks_cells(c), NT, 0, s>>>(face_in(c), nullptr, o, geo_of(c), phys_of(c),
+                                              c->red_part, c->red_cnt, c->ctrl);
 }
 
 void launch_scale_jl(const erem_ctx* c, double sc, cudaStream_t s) {
@@ -2862,13 +2961,23 @@ void launch_scale_jl(const erem_ctx* c, double sc, cudaStream_t s) {
   jc.b0 = nullptr;
   const int nc = c->dim == 3 ? 7 : 5;
   ++c->launches;
-  if (c->prec == EREM_FP32_BULK)
-    k_scale_jl<float, 128><<<blocks_padded(c), NT, 0, s>>>(jc, (float*)c->jl_all, sc, (int)c->Np, nc,
-                                                           c->jrow, c->jl_nodiag ? 1 : 0, c->jl_r0,
-                                                           c->px);
+  const int nb = blocks_padded(c), np = (int)c->Np;
+  if (c->prec == EREM_FP32_BULK) {
+    float* out = (float*)c->jl_all;
+    // the row sums serve the step start of the linear fluid
+    float2* rs = c->phys.fluid_model ? nullptr : c->jrow;
+    if (nc == 7 && c->jl_nodiag)
+      k_scale_jl<float, 128, 7, 1><<<nb, NT, 0, s>>>(jc, out, sc, np, rs, c->jl_r0, c->px);
+    else if (nc == 7)
+      k_scale_jl<float, 128, 7, 0><<<nb, NT, 0, s>>>(jc, out, sc, np, rs, nullptr, c->px);
+    else if (c->jl_nodiag)
+      k_scale_jl<float, 128, 5, 1><<<nb, NT, 0, s>>>(jc, out, sc, np, rs, c->jl_r0, c->px);
+    else
+      k_scale_jl<float, 128, 5, 0><<<nb, NT, 0, s>>>(jc, out, sc, np, rs, nullptr, c->px);
+  } else if (nc == 7)
+    k_scale_jl<double, 64, 7, 0><<<nb, NT, 0, s>>>(jc, (double*)c->jl_all, sc, np, nullptr, nullptr, c->px);
   else
-    k_scale_jl<double, 64><<<blocks_padded(c), NT, 0, s>>>(jc, (double*)c->jl_all, sc, (int)c->Np, nc,
-                                                           nullptr, 0, nullptr, c->px);
+    k_scale_jl<double, 64, 5, 0><<<nb, NT, 0, s>>>(jc, (double*)c->jl_all, sc, np, nullptr, nullptr, c->px);
 }
 
 // Pointers of the interleaved Leja coefficients for kernels of vector width
@@ -2895,6 +3004,11 @@ void launch_rhs(const erem_ctx* c, const double* T, double* G, int set_yinf, cud
   ++c->launches;
   k_rhs<<<blocks_cells(c), NT, 0, s>>>(face_in(c), T, G, geo_of(c), phys_of(c), set_yinf,
                                        c->red_part, c->red_cnt, c->ctrl);
+}
+
+void launch_yinf(const erem_ctx* c, const double* T, cudaStream_t s) {
+  ++c->launches;
+  k_yinf<<<grid_for(c, c->Np / 4), NT, 0, s>>>(T, (int)c->Np, c->red_part, c->red_cnt, c->ctrl);
 }
 
 void launch_sumsq(const erem_ctx* c, const double* x, cudaStream_t s) {
@@ -3122,16 +3236,21 @@ void launch_lincomb(const erem_ctx* c, double* out, double a, const double* x, d
 // afterwards; free again once the CG has converged)
 void launch_pres_faces(const erem_ctx* c, const double* lnk, const double* T, cudaStream_t s) {
   const PresArr a = pres_arr(c);
-  c->launches += 2;
+  c->launches += 3;
   k_mobility<<<blocks_cells(c), NT, 0, s>>>(lnk, T, a.r, geo_of(c), phys_of(c), 0, 0,
                                             &c->ctrl->flags);
   k_pres_faces<<<blocks_cells(c), NT, 0, s>>>(a.r, a, geo_of(c), phys_of(c));
+  k_pres_diag<<<blocks_cells(c), NT, 0, s>>>(a.r, a, geo_of(c), phys_of(c));
 }
 
 void launch_cg_init(const erem_ctx* c, double tol, cudaStream_t s) {
   ++c->launches;
-  k_cg_init<<<blocks_cells(c), NT, 0, s>>>(pres_arr(c), geo_of(c), tol, c->red_part, c->red_cnt,
-                                           c->ctrl);
+  if (c->pc_deg == 1)
+    k_cg_init<1><<<blocks_cells(c), NT, 0, s>>>(pres_arr(c), geo_of(c), tol, c->red_part, c->red_cnt,
+                                                c->ctrl);
+  else
+    k_cg_init<0><<<blocks_cells(c), NT, 0, s>>>(pres_arr(c), geo_of(c), tol, c->red_part, c->red_cnt,
+                                                c->ctrl);
 }
 
 void launch_cg_iter(const erem_ctx* c, int k, cudaStream_t s) {
@@ -3139,9 +3258,9 @@ void launch_cg_iter(const erem_ctx* c, int k, cudaStream_t s) {
   const double* dold = (k & 1) ? a.d1 : a.d0;
   double* dnew = (k & 1) ? a.d0 : a.d1;
   const int nb = blocks_cells(c);
-  ++c->launches;
-  k_cg_dir<double><<<nb, NT, 0, s>>>(a, a.z, dold, dnew, geo_of(c), c->red_part, c->red_cnt,
-                                     c->ctrl);
+  c->launches += 2;
+  k_cg_newdir<double><<<grid_for(c, c->Np / 4), NT, 0, s>>>(a.z, dold, dnew, (int)c->Np, c->ctrl);
+  k_cg_dir<<<nb, NT, 0, s>>>(a, dnew, geo_of(c), c->red_part, c->red_cnt, c->ctrl);
   ++c->launches;
   k_cg_upd<<<nb, NT, 0, s>>>(a, dnew, geo_of(c), c->red_part, c->red_cnt, c->ctrl);
 }
@@ -3325,8 +3444,9 @@ void launch_pcg_iter(const erem_ctx* c, const PcPoly& poly, const float* z, int 
   const double* dold = (k & 1) ? a.d1 : a.d0;
   double* dnew = (k & 1) ? a.d0 : a.d1;
   const int nb = blocks_cells(c);
-  ++c->launches;
-  k_cg_dir<float><<<nb, NT, 0, s>>>(a, z, dold, dnew, geo_of(c), c->red_part, c->red_cnt, c->ctrl);
+  c->launches += 2;
+  k_cg_newdir<float><<<grid_for(c, c->Np / 4), NT, 0, s>>>(z, dold, dnew, (int)c->Np, c->ctrl);
+  k_cg_dir<<<nb, NT, 0, s>>>(a, dnew, geo_of(c), c->red_part, c->red_cnt, c->ctrl);
   ++c->launches;
   k_pcg_upd<<<nb, NT, 0, s>>>(a, dnew, geo_of(c), c->red_part, c->red_cnt, c->ctrl);
   // the next z lands in the same buffer (the preconditioner's sweep count is fixed)
@@ -3335,10 +3455,16 @@ void launch_pcg_iter(const erem_ctx* c, const PcPoly& poly, const float* z, int 
 
 void launch_pres_post(const erem_ctx* c, const double* lnk, const double* T, cudaStream_t s) {
   const PresArr a = pres_arr(c);
+  if (c->phys.fluid_model == 0) {
+    ++c->launches;
+    k_pres_post<0><<<blocks_cells(c), NT, 0, s>>>(lnk, a, geo_of(c), phys_of(c), c->red_part,
+                                                  c->red_cnt, c->ctrl);
+    return;
+  }
   c->launches += 2;
   k_mobility<<<blocks_cells(c), NT, 0, s>>>(lnk, T, a.r, geo_of(c), phys_of(c), 1, 0, nullptr);
-  k_pres_post<<<blocks_cells(c), NT, 0, s>>>(a.r, a.x, geo_of(c), phys_of(c), c->red_part,
-                                             c->red_cnt, c->ctrl);
+  k_pres_post<1><<<blocks_cells(c), NT, 0, s>>>(a.r, a, geo_of(c), phys_of(c), c->red_part,
+                                                c->red_cnt, c->ctrl);
 }
 
 void launch_bicg_init(const erem_ctx* c, const double* b, double sigma, double tol,

@@ -112,6 +112,7 @@ extern "C" erem_status erem_pressure_solve_static(const erem_grid* grid, const e
   v.ax = v.hy * v.hz;
   v.ay = v.hx * v.hz;
   v.az = v.hx * v.hy;
+  v.pc_deg = 1;   // Jacobi
   v.device = dev;
   v.sm_count = sms;
   v.red_blocks = sms * 8 < kMaxBlocks ? sms * 8 : kMaxBlocks;
