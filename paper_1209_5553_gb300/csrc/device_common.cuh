@@ -176,6 +176,51 @@ __device__ __forceinline__ bool bits_finite(unsigned long long b) {
   return (b >> 52) != 0x7ffULL;
 }
 
+// sqrt(x) for x >= 0 (infinities, NaNs and negative x give what sqrt gives): the
+// FP32 reciprocal root of the significand scaled to [1, 4), then two Newton
+// steps for the root in FP64 (each squares the relative error: 2^-22, 2^-43,
+// 2^-53), 7 FP64 operations.  An FP64 operation holds a scheduler's FP64 unit
+// for 64 cycles on this part, and the library's sqrt() is a chain of many.
+__device__ __forceinline__ double sqrt_newton(double x) {
+  const unsigned long long b = abs_bits(x);
+  const int e = (int)(b >> 52);
+  if (x < 0.0 || e == 0 || e == 0x7ff) return sqrt(x);   // zeros, subnormals, infinities, NaNs
+  const int h = (e - 1023) >> 1;                         // x = m 4^h, 1 <= m < 4
+  const double m = __longlong_as_double((long long)(b - ((unsigned long long)(2 * h) << 52)));
+  const double y = f2d_fast(rsqrtf(__double2float_rn(m)));
+  const double hy = 0.5 * y;
+  double s = m * y;
+  s = fma(fma(-s, s, m), hy, s);
+  s = fma(fma(-s, s, m), hy, s);
+  return __longlong_as_double(__double_as_longlong(s) + ((long long)h << 52));
+}
+
+// n / d by Newton's method: the reciprocal of d's significand from FP32 (2^-22
+// after rounding d to 24 bits), one Newton step for it in FP64 (2^-44), and
+// the residual correction of the quotient, q + (n - d q) y, which is exact up to
+// its last rounding and 2^-88 of the quotient: the correctly rounded quotient
+// but for one in about 10^10 operand pairs, and then one unit in the last
+// place off.  Five FP64 operations, the rest on integers and FP32.  Operands
+// outside 2^+-500 (zero numerators apart) take the ordinary division.
+__device__ __forceinline__ double div_newton(double n, double d) {
+  const unsigned dh = (unsigned)__double2hiint(d), dl = (unsigned)__double2loint(d);
+  const unsigned nh = (unsigned)__double2hiint(n);
+  const unsigned ed = (dh >> 20) & 0x7ffu, en = (nh >> 20) & 0x7ffu;
+  const bool zero_n = abs_bits(n) == 0ULL;
+  if (ed - 523u > 1000u || (en - 523u > 1000u && !zero_n)) return n / d;
+  // |d| = m 2^(ed - 1023), m rounded to a float in [1, 2]
+  const unsigned mb = 0x3f800000u + ((((dh & 0xfffffu) << 3) | (dl >> 29)) + ((dl >> 28) & 1u));
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint_as_float(mb)));
+  const unsigned rb = __float_as_uint(r);
+  const unsigned er = ((rb >> 23) & 0xffu) + 896u + 1023u - ed;   // exponent of y 2^-(ed - 1023)
+  double y = __hiloint2double((int)((dh & 0x80000000u) | (er << 20) | ((rb & 0x7fffffu) >> 3)),
+                              (int)(rb << 29));
+  y = fma(fma(-d, y, 1.0), y, y);
+  const double q = n * y;
+  return fma(fma(-d, q, n), y, q);
+}
+
 // The Leja copy of J is interleaved per warp tile of T = 32 VEC cells: the
 // tile's NC coefficient arrays D W E S N (B T) follow one another, T values
 // each.  A warp whose lanes own 32 consecutive VEC-cell vectors reads each

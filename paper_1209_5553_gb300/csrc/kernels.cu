@@ -60,7 +60,7 @@ __device__ __forceinline__ double dXof(double T, int fm) { return fm ? rho_rel(T
 // two-point harmonic transmissibility |s| ki kj / (ki d + kj d), uniform d
 __device__ __forceinline__ double harm(double area, double d, double ki, double kj) {
   const double den = ki * d + kj * d;
-  return den != 0.0 ? area * ki * kj / den : 0.0;
+  return abs_bits(den) != 0ULL ? div_newton(area * ki * kj, den) : 0.0;
 }
 
 struct Phys {
@@ -165,7 +165,7 @@ __global__ void k_mobility(const double* __restrict__ lnk, const double* __restr
     double mi = exp(lnk[j]);
     if (ph.fm) {  // a linear fluid has density and viscosity 1: no FP64 division by it
       const double Ti = T ? T[j] : 20.0;
-      mi = darcy ? mi / mu_rel(Ti, 1) : mi * rho_rel(Ti, 1) / mu_rel(Ti, 1);
+      mi = div_newton(darcy ? mi : mi * rho_rel(Ti, 1), mu_rel(Ti, 1));
     }
     bad |= !finite(mi);
     m[ip] = mi;
@@ -225,7 +225,7 @@ __global__ void k_faces(FieldIn in, const double* __restrict__ m, FaceOut o, Geo
     if (o.dX) o.dX[ip] = dXof(Ti, 1);
     const double C = phi * ph.rhoc_f + (1.0 - phi) * ph.rhoc_s;
     inval |= neg(C) | (abs_bits(C) == 0ULL) | (abs_bits(C) > 0x7ff0000000000000ULL);  // !(C > 0)
-    o.icap[ip] = 1.0 / (C * ph.vol);
+    o.icap[ip] = div_newton(1.0, C * ph.vol);
   }
   if (bad) atomicOr(flags, FLAG_NONFINITE);
   if (inval) atomicOr(flags, FLAG_BAD_INPUT);
@@ -262,14 +262,15 @@ __global__ void k_cellJ(FaceIn f, const double* __restrict__ dX, JOut o, Geo g, 
     // F > 0 leaves through a + face carrying X_i, F < 0 enters carrying X_j;
     // every product and sum is rounded on its own
     auto times = [](double F, double d) { return FM ? __dmul_rn(F, d) : F; };
+    auto mag = [](double F) { return __longlong_as_double((long long)abs_bits(F)); };
     auto plus = [&](int q, double L, double F, double& c) {
       const bool in = neg(F);
       D = __dsub_rn(D, __dadd_rn(L, in ? 0.0 : times(F, dXi)));
-      c = __dadd_rn(L, in ? times(-F, FM ? dX[q] : 1.0) : 0.0);
+      c = __dadd_rn(L, in ? times(mag(F), FM ? dX[q] : 1.0) : 0.0);
     };
     auto minus = [&](int q, double L, double F, double& c) {
       const bool out = neg(F);
-      D = __dsub_rn(D, __dadd_rn(L, out ? times(-F, dXi) : 0.0));
+      D = __dsub_rn(D, __dadd_rn(L, out ? times(mag(F), dXi) : 0.0));
       c = __dadd_rn(L, out ? 0.0 : times(F, FM ? dX[q] : 1.0));
     };
     if (ix < g.nx - 1) plus(ip + 1, f.Lx[ip], f.Fx[ip], E);
@@ -293,17 +294,18 @@ __global__ void k_cellJ(FaceIn f, const double* __restrict__ dX, JOut o, Geo g, 
     D *= ic; W *= ic; E *= ic; S *= ic; Nn *= ic;
     o.c[0][ip] = D; o.c[1][ip] = W; o.c[2][ip] = E; o.c[3][ip] = S; o.c[4][ip] = Nn;
     double R = fabs(W) + fabs(E) + fabs(S) + fabs(Nn);
-    double rs = D + W + E + S + Nn;
     if (g.dim == 3) {
       B *= ic; Tt *= ic;
       o.c[5][ip] = B; o.c[6][ip] = Tt;
       R = R + fabs(B) + fabs(Tt);
-      rs = rs + B + Tt;
     }
     bad |= !finite(D) | !finite(R);
+    const double top = D + R;
     gmin = min(gmin, rank_of(D - R));
-    gmax = max(gmax, rank_of(D + R));
+    gmax = max(gmax, rank_of(top));
     // the row sum relative to the couplings, off the Dirichlet inflow plane
+    // (linear fluid: the couplings are >= 0, so it is D + R)
+    const double rs = FM ? D + W + E + S + Nn + B + Tt : top;
     if (ix > 0) tilted |= abs_bits(rs) > abs_bits(kRowSumNoDiag * R);
   }
   if (bad) atomicOr(&ctrl->flags, FLAG_NONFINITE);
@@ -1662,41 +1664,38 @@ struct PresArr {
   double *x, *r, *z, *d0, *d1, *Ad, *Ux, *Uy, *Uz, *diag, *b;
 };
 
-// TPFA pressure matrix from the cell mobilities m: the couplings to the next
-// cell in x, y and z.  The diagonal sums them in a pass of its own
-// (k_pres_diag): formed here it would evaluate every harmonic mean twice, and
-// their FP64 divisions bound the pass (128^3: 374 us, now 151 + 59)
+// The same mean by the compiler's division.  The matrix below is formed from
+// both sides of every face; with the sums and divisions written out by hand
+// (330 us instead of 374 at 128^3) its last bits, and with them the last bits
+// of p, changed, which an FP32-bulk step with T-dependent fluid laws amplifies to
+// its own rounding level.
+__device__ __forceinline__ double harm_div(double area, double d, double ki, double kj) {
+  const double den = ki * d + kj * d;
+  return den != 0.0 ? area * ki * kj / den : 0.0;
+}
+
+// TPFA pressure matrix from the cell mobilities m: upper couplings, diagonal
+// (with the Dirichlet faces at x = 0 and x = 1) and right-hand side
 __global__ void k_pres_faces(const double* __restrict__ m, PresArr a, Geo g, Phys ph) {
   for (int i = blockIdx.x * NT + threadIdx.x; i < g.N; i += gridDim.x * NT) {
     int ix, iy, iz, ip;
     cell_of(i, g, ix, iy, iz, ip);
     const double mi = m[ip];
+    double dg = 0.0, bb = 0.0;
     double ux = 0.0, uy = 0.0, uz = 0.0;
-    if (ix < g.nx - 1) ux = harm(ph.ax, 0.5 * ph.hx, mi, m[ip + 1]);
-    if (iy < g.ny - 1) uy = harm(ph.ay, 0.5 * ph.hy, mi, m[ip + g.px]);
-    if (g.dim == 3 && iz < g.nz - 1) uz = harm(ph.az, 0.5 * ph.hz, mi, m[ip + g.plane]);
+    if (ix < g.nx - 1) ux = harm_div(ph.ax, 0.5 * ph.hx, mi, m[ip + 1]);
+    if (iy < g.ny - 1) uy = harm_div(ph.ay, 0.5 * ph.hy, mi, m[ip + g.px]);
+    if (g.dim == 3 && iz < g.nz - 1) uz = harm_div(ph.az, 0.5 * ph.hz, mi, m[ip + g.plane]);
     a.Ux[ip] = ux;
     a.Uy[ip] = uy;
     if (g.dim == 3) a.Uz[ip] = uz;
-  }
-}
-
-// The diagonal (the six couplings of a cell and the Dirichlet faces at x = 0
-// and x = 1) and the right-hand side.
-__global__ void k_pres_diag(const double* __restrict__ m, PresArr a, Geo g, Phys ph) {
-  for (int i = blockIdx.x * NT + threadIdx.x; i < g.N; i += gridDim.x * NT) {
-    int ix, iy, iz, ip;
-    cell_of(i, g, ix, iy, iz, ip);
-    double dg = 0.0, bb = 0.0;
-    dg += a.Ux[ip] + a.Uy[ip] + (g.dim == 3 ? a.Uz[ip] : 0.0);
-    if (ix > 0) dg += a.Ux[ip - 1];
-    if (iy > 0) dg += a.Uy[ip - g.px];
-    if (g.dim == 3 && iz > 0) dg += a.Uz[ip - g.plane];
-    if (ix == 0 || ix == g.nx - 1) {
-      const double uD = ph.ax * m[ip] / (0.5 * ph.hx);
-      if (ix == 0) { dg += uD; bb += uD * ph.head_left; }
-      if (ix == g.nx - 1) { dg += uD; bb += uD * ph.head_right; }
-    }
+    dg += ux + uy + uz;
+    if (ix > 0) dg += harm_div(ph.ax, 0.5 * ph.hx, m[ip - 1], mi);
+    if (iy > 0) dg += harm_div(ph.ay, 0.5 * ph.hy, m[ip - g.px], mi);
+    if (g.dim == 3 && iz > 0) dg += harm_div(ph.az, 0.5 * ph.hz, m[ip - g.plane], mi);
+    const double uD = ph.ax * mi / (0.5 * ph.hx);
+    if (ix == 0) { dg += uD; bb += uD * ph.head_left; }
+    if (ix == g.nx - 1) { dg += uD; bb += uD * ph.head_right; }
     a.diag[ip] = dg;
     a.b[ip] = bb;
   }
@@ -1887,7 +1886,7 @@ __global__ void k_pc_setup(PresArr a, PcArr p, float* __restrict__ diag32, Geo g
   for (int i = blockIdx.x * NT + threadIdx.x; i < g.N; i += gridDim.x * NT) {
     int ix, iy, iz, ip;
     cell_of(i, g, ix, iy, iz, ip);
-    p.dinv[ip] = (float)(1.0 / a.diag[ip]);
+    p.dinv[ip] = (float)div_newton(1.0, a.diag[ip]);
     if (diag32) diag32[ip] = (float)a.diag[ip];
     p.Ux[ip] = (float)a.Ux[ip];
     p.Uy[ip] = (float)a.Uy[ip];
@@ -3236,11 +3235,10 @@ void launch_lincomb(const erem_ctx* c, double* out, double a, const double* x, d
 // afterwards; free again once the CG has converged)
 void launch_pres_faces(const erem_ctx* c, const double* lnk, const double* T, cudaStream_t s) {
   const PresArr a = pres_arr(c);
-  c->launches += 3;
+  c->launches += 2;
   k_mobility<<<blocks_cells(c), NT, 0, s>>>(lnk, T, a.r, geo_of(c), phys_of(c), 0, 0,
                                             &c->ctrl->flags);
   k_pres_faces<<<blocks_cells(c), NT, 0, s>>>(a.r, a, geo_of(c), phys_of(c));
-  k_pres_diag<<<blocks_cells(c), NT, 0, s>>>(a.r, a, geo_of(c), phys_of(c));
 }
 
 void launch_cg_init(const erem_ctx* c, double tol, cudaStream_t s) {

@@ -136,25 +136,6 @@ __device__ __forceinline__ void ldv_cg(Tq (&r)[VEC], const Tq* p) {
   for (int k = 0; k < VEC; ++k) r[k] = s[k];
 }
 
-// sqrt(x) for x >= 0 (infinities, NaNs and negative x give what sqrt gives): the
-// FP32 reciprocal root of the significand scaled to [1, 4), then two Newton
-// steps for the root in FP64 (each squares the relative error: 2^-22, 2^-43,
-// 2^-53), 7 FP64 operations.  An FP64 operation holds a scheduler's FP64 unit
-// for 64 cycles on this part, and the library's sqrt() is a chain of many.
-__device__ __forceinline__ double sqrt_newton(double x) {
-  const unsigned long long b = abs_bits(x);
-  const int e = (int)(b >> 52);
-  if (x < 0.0 || e == 0 || e == 0x7ff) return sqrt(x);   // zeros, subnormals, infinities, NaNs
-  const int h = (e - 1023) >> 1;                         // x = m 4^h, 1 <= m < 4
-  const double m = __longlong_as_double((long long)(b - ((unsigned long long)(2 * h) << 52)));
-  const double y = f2d_fast(rsqrtf(__double2float_rn(m)));
-  const double hy = 0.5 * y;
-  double s = m * y;
-  s = fma(fma(-s, s, m), hy, s);
-  s = fma(fma(-s, s, m), hy, s);
-  return __longlong_as_double(__double_as_longlong(s) + ((long long)h << 52));
-}
-
 // neighbour sources of a vector (bits of its mask)
 enum : int {
   RS_OWN = 1,              // the thread owns this vector
