@@ -496,7 +496,9 @@ erem_status leja_interp(erem_ctx* c, const double* u, const double* fused_T, int
   // before it (k_leja_term_lag), so the launch after the stopping term is
   // needed too: it completes P
   // resident launches are lagged in the same way
-  const int lag = res ? kResLag : (c->term_lag && !slot0) ? 1 : 0;
+  // large 3D FP32-bulk grids, untaped: two terms per pass
+  const bool pair = !res && !slot0 && leja_pair_fits(c);
+  const int lag = res ? kResLag : (c->term_lag && !slot0 && !pair) ? 1 : 0;
   if (lag) c->last_lag = true;
   int m = 1, qin = 0;
   int chunk = res ? kResTerms : forced ? forced + lag : std::max(4, c->last_degree + 2 + lag);
@@ -507,6 +509,7 @@ erem_status leja_interp(erem_ctx* c, const double* u, const double* fused_T, int
   std::vector<std::pair<int, int>> chunks;
   while (true) {
     const int last = (forced ? forced : *M_avail) + lag;
+    if (pair) chunk += chunk & 1;
     const int end = std::min(last, m + chunk - 1);
     if (o.time_terms) cudaEventRecord(c->ev[2 * chunks.size()], s);
     if (res) {
@@ -514,7 +517,11 @@ erem_status leja_interp(erem_ctx* c, const double* u, const double* fused_T, int
                                    slot0 ? (forced ? forced : end) : 0, slot0, qbytes, cg, s));
       qin = end & 1;
     }
-    for (int mm = m; !res && mm <= end; ++mm) {
+    for (int mm = m; pair && mm <= end; mm += 2) {
+      EREM_CUDA(c, launch_leja_pair(c, mm, end, qin, cg, s));
+      qin ^= 1;
+    }
+    for (int mm = m; !res && !pair && mm <= end; ++mm) {
       if (slot0)
         launch_leja_term_ptr(c, mm, slot0 + (size_t)(mm - 1) * qbytes, slot0 + (size_t)mm * qbytes,
                              cg, s);
@@ -577,13 +584,13 @@ erem_status leja_interp(erem_ctx* c, const double* u, const double* fused_T, int
       if (cudaEventElapsedTime(&ms, c->ev[2 * j], c->ev[2 * j + 1]) == cudaSuccess) {
         tt->ms += ms;
         tt->terms += std::min(last, *degree) - first + 1;
-        tt->launches += res ? 1 : last - first + 1;
+        tt->launches += res ? 1 : pair ? (last - first + 2) / 2 : last - first + 1;
       }
     }
   }
   c->last_degree = *degree;
   if (!lag && *degree % 2 == 0) {  // q_M: the tape slot, or the ping-pong buffer of m's parity
-    const void* qM = slot0 ? (const void*)(slot0 + (size_t)*degree * qbytes) : c->q[*degree & 1];
+    const void* qM = slot0 ? (const void*)(slot0 + (size_t)*degree * qbytes) : c->q[(pair ? *degree / 2 : *degree) & 1];
     if (fix) *fix = PFixHost{qM, *degree};
     else launch_pfix(c, qM, *degree, s);
   }
@@ -1364,6 +1371,11 @@ erem_status erem_create(const erem_grid* grid, const erem_physics* phys, erem_pr
     coop = 0;
   }
   c->res_ok = coop != 0 && !std::getenv("EREM_TERM_LAG");
+  c->pair_ok = c->smem_optin > 0 && !std::getenv("EREM_TERM_LAG");
+  if (const char* e = std::getenv("EREM_TERM_PAIR")) {  // tuning override: pairs, also on grids that fit on the chip
+    c->pair_ok = c->smem_optin > 0 && std::atoi(e) != 0;
+    if (c->pair_ok) c->res_ok = false;
+  }
   c->term_lag = Np <= kLagCells;
   if (const char* e = std::getenv("EREM_TERM_LAG")) c->term_lag = std::atoi(e) != 0;  // override
   const size_t np = (size_t)Np, nf = (size_t)g.ny * g.nz;

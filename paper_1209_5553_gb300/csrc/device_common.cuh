@@ -245,10 +245,12 @@ __device__ __forceinline__ size_t leja_off(int i, int nc) {
 __device__ void stop_test(Ctrl* c, int m, double dm, double S) {
   const StopParams sp = c->sp;
   const double scal = sp.tol_a + sp.tol_r * c->yinf;
-  const double e = fabs(sp.delta * dm) / scal * sqrt(S / sp.ncells);
+  // one thread on the critical path of a launch: the library's division and
+  // root are chains of a thousand cycles and more
+  const double e = div_newton(fabs(sp.delta * dm), scal) * sqrt_newton(div_newton(S, sp.ncells));
   c->e[m] = e;
   c->m_last = m;
-  if (!isfinite(e)) {
+  if (!bits_finite(abs_bits(e))) {
     c->nonfinite = 1;
     c->done = 1;
     return;
@@ -256,7 +258,7 @@ __device__ void stop_test(Ctrl* c, int m, double dm, double S) {
   const int lo = max(1, m - sp.window + 1);
   double mean = 0.0;
   for (int k = lo; k <= m; ++k) mean += c->e[k];
-  mean /= (double)(m - lo + 1);
+  mean = div_newton(mean, (double)(m - lo + 1));
   c->err = mean;
   if (sp.replay) return;
   if (sp.pow10 * mean < 1.0) {

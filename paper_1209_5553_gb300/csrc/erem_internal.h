@@ -197,6 +197,7 @@ struct erem_ctx {
   // resident Leja kernel (leja_resident.cu): messages and partial sums of its
   // CTAs (allocated on first use), and the number its next launch counts from
   bool res_ok = false;
+  bool pair_ok = false;   // two terms per pass on large 3D grids (leja_pair.cu)
   int smem_optin = 0;             // shared memory a CTA may have
   int res_hy = 0, res_hz = 0;     // rows of a CTA's block (0: not chosen yet)
   void* res_msg = nullptr;
@@ -410,6 +411,9 @@ size_t res_msg_bytes(const erem_ctx* c);
 size_t res_part_bytes(const erem_ctx* c);
 cudaError_t launch_leja_res(erem_ctx* c, int m0, int m1, int ndd, int keep_q, int tape_to, char* tape,
                             size_t qbytes, double cg, cudaStream_t s);
+// Pair form (leja_pair.cu): terms m (odd) and m + 1 in one pass.
+bool leja_pair_fits(const erem_ctx* c);
+cudaError_t launch_leja_pair(const erem_ctx* c, int m, int m_end, int qin, double cg, cudaStream_t s);
 void launch_lincomb(const erem_ctx* c, double* out, double a, const double* x, double b,
                     const double* y, cudaStream_t s);
 
