@@ -12,6 +12,8 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
+#include <queue>
 #include <string>
 #include <thread>
 #include <vector>
@@ -19,6 +21,17 @@
 #include "erem_internal.h"
 
 using namespace erem;
+
+// One launch of a run: `count` members of the queue order from `first`, on
+// clusters of cs CTAs, with the members' working sets in shared memory (res)
+// or in L2.
+struct EnsLaunch {
+  bool res = false;
+  int cs = 0, clusters = 0, first = 0, count = 0;
+  bool operator==(const EnsLaunch& o) const {
+    return res == o.res && cs == o.cs && clusters == o.clusters && first == o.first && count == o.count;
+  }
+};
 
 struct erem_ens {
   int n = 0;
@@ -61,7 +74,9 @@ struct erem_ens {
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t run_exec = nullptr;
   EnsRun run_key{};
-  int key_cs = 0, key_clusters = 0;
+  std::vector<EnsLaunch> key_launches;
+  std::vector<EnsLaunch> launches;   // of the next run
+  int fit_res[5] = {-1, -1, -1, -1, -1}, fit_l2[5] = {-1, -1, -1, -1, -1};   // clusters of 1 << k CTAs at once
   bool graph_ok = true;             // false after a failed capture: direct launches
 
   // statistics of the last run
@@ -70,6 +85,8 @@ struct erem_ens {
 };
 
 namespace {
+
+constexpr int kEnsLaunches = 8;   // launches of a run, at most
 
 erem_status efail(erem_ens* E, erem_status st, const std::string& m) {
   if (E) E->err = m;
@@ -193,7 +210,7 @@ erem_status build(erem_ens* E) {
   ENS_TRY(ens_alloc(E, &E->dd_d, dd.size()));
   ENS_TRY(ens_alloc(E, &E->xi_d, (size_t)M + 1));
   ENS_TRY(ens_alloc(E, &E->order_d, (size_t)E->n));
-  ENS_TRY(ens_alloc(E, &E->next_d, (size_t)1));
+  ENS_TRY(ens_alloc(E, &E->next_d, (size_t)kEnsLaunches));
   if (cudaMallocHost((void**)&E->st_h, sizeof(EnsState) * E->n) != cudaSuccess ||
       cudaMallocHost((void**)&E->order_h, sizeof(int) * E->n) != cudaSuccess)
     return efail(E, EREM_ENOMEM, "cudaMallocHost of the ensemble tables failed");
@@ -229,23 +246,12 @@ erem_status build(erem_ens* E) {
     m.sp.replay = 0;
     m.dt = E->dt[e];
     m.cg = c->cfoc / c->gam;
+    m.rsqrt_n = 1.0 / std::sqrt((double)c->N);
   }
   ENS_CUDA(E, cudaMemcpy(E->mem_d, mem.data(), sizeof(EnsMember) * E->n, cudaMemcpyHostToDevice));
   ENS_CUDA(E, cudaMemcpy(E->dd_d, dd.data(), sizeof(double) * dd.size(), cudaMemcpyHostToDevice));
   ENS_CUDA(E, cudaMemcpy(E->xi_d, xi.data(), sizeof(double) * (M + 1), cudaMemcpyHostToDevice));
   E->built = true;
-  return EREM_OK;
-}
-
-// Cluster size of the next run and the clusters that fit at once.
-erem_status cluster_shape(erem_ens* E, int* cs, int* clusters) {
-  *cs = E->cfg.cluster_ctas ? E->cfg.cluster_ctas : (E->tuned_cs ? E->tuned_cs : 8);
-  int fit = 0;
-  ENS_CUDA(E, ens_max_clusters(E->prec, *cs, &fit));
-  if (fit < 1)
-    return efail(E, EREM_ECUDA, "a cluster of " + std::to_string(*cs) + " CTAs does not fit the device");
-  if (E->cfg.max_clusters > 0) fit = std::min(fit, E->cfg.max_clusters);
-  *clusters = std::min(fit, E->n);
   return EREM_OK;
 }
 
@@ -258,6 +264,163 @@ double member_weight(const erem_ens* E, int e) {
   return rate * ((double)c->Np + 16384.0);
 }
 
+// Clusters of cs CTAs that run at once (0: none).
+int fit_clusters(erem_ens* E, int cs, bool res) {
+  int k = 0;
+  while ((1 << k) < cs) ++k;
+  int& f = res ? E->fit_res[k] : E->fit_l2[k];
+  if (f < 0) {
+    const cudaError_t e = res ? ens_res_max_clusters(E->prec, cs, E->ctx[0]->smem_optin, &f)
+                              : ens_max_clusters(E->prec, cs, &f);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      f = 0;
+    }
+  }
+  return E->cfg.max_clusters > 0 ? std::min(f, E->cfg.max_clusters) : f;
+}
+
+bool fits_resident(const erem_ens* E, int e, int cs) {
+  if (const char* v = std::getenv("EREM_ENS_RESIDENT"))  // tuning override: 0 keeps every member in L2
+    if (std::atoi(v) == 0) return false;
+  const erem_ctx* c = E->ctx[e];
+  return ens_res_fits(E->prec, cs, c->ny, c->px, c->jl_nodiag, c->smem_optin);
+}
+
+// Passes per step of member e: of its last run, else the width of its
+// spectral interval as a proxy for the Leja degree.
+double member_rate(const erem_ens* E, int e) {
+  return E->pass_rate[e] > 0.0 ? E->pass_rate[e] : 1.0 + E->ctx[e]->gam;
+}
+
+// Time of one pass of member e on cs CTAs, us, measured on 64^2 to 480^2
+// members and clusters of 2 to 16.  In shared memory: the barrier and the
+// control step, then the band's vectors (FP64 pipe: one operation per cell in
+// FP32-bulk, eight in FP64).  From L2: the same, then the load latency of the
+// sweep.
+double pass_time(const erem_ens* E, int e, int cs, bool res) {
+  const erem_ctx* c = E->ctx[e];
+  const bool f32 = E->prec == EREM_FP32_BULK;
+  const double nvb = (double)((c->ny + cs - 1) / cs) * (c->px / (f32 ? 4 : 2));
+  if (res) return f32 ? 2.5 + 0.00085 * nvb : 2.7 + 0.0036 * nvb;
+  return f32 ? 4.0 + 0.0032 * nvb : 5.0 + 0.0043 * nvb;
+}
+
+// Time of the given members in one launch: the queue played through, heaviest
+// first over the clusters that run at once, and from L2 at least the rate of
+// the whole chip (110 cells per ns in FP32-bulk, 41 in FP64).
+double launch_time(erem_ens* E, const std::vector<int>& who, int cs, bool res) {
+  const int slots = fit_clusters(E, cs, res);
+  if (slots < 1) return 1e300;
+  double cells = 0.0;
+  std::vector<double> t(who.size());
+  for (size_t k = 0; k < who.size(); ++k) {
+    const double r = member_rate(E, who[k]);
+    t[k] = r * pass_time(E, who[k], cs, res);
+    cells += r * (double)E->ctx[who[k]]->Np;
+  }
+  std::sort(t.begin(), t.end(), std::greater<double>());
+  std::priority_queue<double, std::vector<double>, std::greater<double>> busy;
+  double end = 0.0;
+  for (size_t k = 0; k < t.size(); ++k) {
+    double at = 0.0;
+    if ((int)k >= slots) {
+      at = busy.top();
+      busy.pop();
+    }
+    busy.push(at + t[k]);
+    end = std::max(end, at + t[k]);
+  }
+  return res ? end : std::max(end, cells / (E->prec == EREM_FP32_BULK ? 110e3 : 41e3));
+}
+
+// The launches of the next run and its queue order.  A given (or tuned)
+// cluster size takes one launch for the members that fit on such a cluster's
+// shared memory and one for the rest.  Otherwise the members are split by the
+// smallest cluster they fit on, neighbouring classes share a launch, and each
+// launch takes the form (shared memory or L2) and the cluster size by which the
+// whole run is shortest.
+erem_status plan_run(erem_ens* E) {
+  const int fixed = E->cfg.cluster_ctas ? E->cfg.cluster_ctas : E->tuned_cs;
+  E->launches.clear();
+  std::vector<std::pair<double, int>> w(E->n);
+  for (int e = 0; e < E->n; ++e) w[e] = {member_weight(E, e), e};
+  std::stable_sort(w.begin(), w.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
+  int pos = 0;
+  auto add = [&](bool res, int cs, const std::vector<char>& in) -> erem_status {
+    EnsLaunch L;
+    L.res = res;
+    L.cs = cs;
+    L.first = pos;
+    for (const auto& x : w)
+      if (in[x.second]) E->order_h[pos++] = x.second;
+    L.count = pos - L.first;
+    if (L.count == 0) return EREM_OK;
+    const int fit = fit_clusters(E, cs, res);
+    if (fit < 1)
+      return efail(E, EREM_ECUDA, "a cluster of " + std::to_string(cs) + " CTAs does not fit the device");
+    L.clusters = std::min(fit, L.count);
+    E->launches.push_back(L);
+    return EREM_OK;
+  };
+  std::vector<char> in(E->n, 0), rest(E->n, 0);
+  if (fixed) {
+    const bool any = fit_clusters(E, fixed, true) > 0;
+    for (int e = 0; e < E->n; ++e) {
+      in[e] = any && fits_resident(E, e, fixed);
+      rest[e] = !in[e];
+    }
+    ENS_TRY(add(true, fixed, in));
+    return add(false, fixed, rest);
+  }
+  // class k: the smallest cluster of 2 << k CTAs the member fits on
+  std::vector<int> cls(E->n, 4);
+  for (int e = 0; e < E->n; ++e)
+    for (int k = 3; k >= 0; --k)
+      if (fit_clusters(E, 2 << k, true) > 0 && fits_resident(E, e, 2 << k)) cls[e] = k;
+  // best[k]: the shortest time of classes < k, the last launch being [from, k)
+  double best[6] = {0.0};
+  int from[6] = {0}, size[6] = {0};
+  bool resident[6] = {false};
+  std::vector<int> who;
+  for (int k = 1; k <= 5; ++k) {
+    best[k] = 1e300;
+    for (int f = 0; f < k; ++f) {
+      who.clear();
+      for (int e = 0; e < E->n; ++e)
+        if (cls[e] >= f && cls[e] < k) who.push_back(e);
+      for (int res = 0; res < 2; ++res)
+        for (int c = 1; c <= 4; ++c) {
+          // the largest class needs clusters of 2 << (k - 1); from L2, clusters of
+          // eight, or of 16 where they all run at once
+          if (res ? c < k : c < 3 || (c == 4 && (int)who.size() > fit_clusters(E, 16, false))) continue;
+          const double t = best[f] + (who.empty() ? 0.0 : launch_time(E, who, 1 << c, res != 0));
+          if (t < best[k]) {
+            best[k] = t;
+            from[k] = f;
+            size[k] = 1 << c;
+            resident[k] = res != 0;
+          }
+        }
+    }
+    if (best[k] >= 1e300) return efail(E, EREM_ECUDA, "no cluster size fits the device");
+  }
+  // one launch from L2 on clusters of eight is the rule for every ensemble: the
+  // plan replaces it where it promises more than the estimates' own error
+  who.resize(E->n);
+  for (int e = 0; e < E->n; ++e) who[e] = e;
+  if (best[5] > 0.8 * launch_time(E, who, 8, false)) {
+    from[5] = 0;
+    size[5] = 8;
+    resident[5] = false;
+  }
+  for (int k = 5; k > 0; k = from[k]) {
+    for (int e = 0; e < E->n; ++e) in[e] = cls[e] >= from[k] && cls[e] < k;
+    ENS_TRY(add(resident[k], size[k], in));
+  }
+  return EREM_OK;
+}
+
 bool same_run(const EnsRun& a, const EnsRun& b) {
   return a.mem == b.mem && a.st == b.st && a.order == b.order && a.next == b.next && a.xi == b.xi &&
          a.n == b.n && a.nlev == b.nlev && a.mmax == b.mmax && a.restart == b.restart &&
@@ -265,15 +428,23 @@ bool same_run(const EnsRun& a, const EnsRun& b) {
 }
 
 // The device work of a run, in stream order: the member states and the queue
-// order up from pinned host memory, the queue position reset, the persistent
-// launch, the states back.  The copies read and write the pinned buffers when
+// order up from pinned host memory, the queue positions reset, the persistent
+// launches, the states back.  The copies read and write the pinned buffers when
 // they execute, so one capture serves every run with the same descriptor.
-cudaError_t enqueue_run(erem_ens* E, const EnsRun& R, int cs, int clusters, cudaStream_t s) {
+cudaError_t enqueue_run(erem_ens* E, const EnsRun& R, cudaStream_t s) {
   cudaError_t e = cudaMemcpyAsync(E->st_d, E->st_h, sizeof(EnsState) * E->n, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(E->order_d, E->order_h, sizeof(int) * E->n, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(E->next_d, 0, sizeof(unsigned), s);
-  if (e == cudaSuccess) e = launch_ens_cluster(R, E->prec, cs, clusters, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(E->next_d, 0, sizeof(unsigned) * kEnsLaunches, s);
+  for (size_t k = 0; k < E->launches.size() && e == cudaSuccess; ++k) {
+    const EnsLaunch& L = E->launches[k];
+    EnsRun r = R;
+    r.order = R.order + L.first;
+    r.n = L.count;
+    r.next = R.next + k;
+    e = L.res ? launch_ens_resident(r, E->prec, L.cs, L.clusters, E->ctx[0]->smem_optin, s)
+              : launch_ens_cluster(r, E->prec, L.cs, L.clusters, s);
+  }
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(E->st_h, E->st_d, sizeof(EnsState) * E->n, cudaMemcpyDeviceToHost, s);
   return e;
@@ -282,7 +453,7 @@ cudaError_t enqueue_run(erem_ens* E, const EnsRun& R, int cs, int clusters, cuda
 // Capture the run on the ensemble's own stream (a legacy default stream
 // cannot be captured) and instantiate it; on any failure the ensemble keeps
 // to direct launches.
-void capture_run(erem_ens* E, const EnsRun& R, int cs, int clusters) {
+void capture_run(erem_ens* E, const EnsRun& R) {
   if (!E->cap_stream && cudaStreamCreateWithFlags(&E->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
     cudaGetLastError();
     E->cap_stream = nullptr;
@@ -295,7 +466,7 @@ void capture_run(erem_ens* E, const EnsRun& R, int cs, int clusters) {
     E->graph_ok = false;
     return;
   }
-  const cudaError_t e = enqueue_run(E, R, cs, clusters, E->cap_stream);
+  const cudaError_t e = enqueue_run(E, R, E->cap_stream);
   const cudaError_t ee = cudaStreamEndCapture(E->cap_stream, &g);
   cudaGraphExec_t x = nullptr;
   if (e != cudaSuccess || ee != cudaSuccess || !g || cudaGraphInstantiate(&x, g, 0) != cudaSuccess) {
@@ -307,8 +478,7 @@ void capture_run(erem_ens* E, const EnsRun& R, int cs, int clusters) {
   cudaGraphDestroy(g);
   E->run_exec = x;
   E->run_key = R;
-  E->key_cs = cs;
-  E->key_clusters = clusters;
+  E->key_launches = E->launches;
 }
 
 // One run: every member advances `steps` steps, one launch of the batched
@@ -318,8 +488,7 @@ void capture_run(erem_ens* E, const EnsRun& R, int cs, int clusters) {
 // at twice the substeps, as erem_step splits a step whose interpolation
 // failed.
 erem_status run(erem_ens* E, int steps, cudaStream_t s) {
-  int cs = 0, clusters = 0;
-  ENS_TRY(cluster_shape(E, &cs, &clusters));
+  ENS_TRY(plan_run(E));
   const bool keep = E->cfg.substep_policy == EREM_ENS_KEEP_SUBSTEPS;
   for (int e = 0; e < E->n; ++e) {
     EnsState& st = E->st_h[e];
@@ -328,11 +497,6 @@ erem_status run(erem_ens* E, int steps, cudaStream_t s) {
     st.level = std::min(keep ? E->level_start[e] : 0, E->nlev - 1);
     st.target = steps;
   }
-  std::vector<std::pair<double, int>> w(E->n);
-  for (int e = 0; e < E->n; ++e) w[e] = {member_weight(E, e), e};
-  std::stable_sort(w.begin(), w.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
-  for (int k = 0; k < E->n; ++k) E->order_h[k] = w[k].second;
-
   EnsRun R{};
   R.mem = E->mem_d;
   R.st = E->st_d;
@@ -349,16 +513,15 @@ erem_status run(erem_ens* E, int steps, cudaStream_t s) {
     if (b >= 1) R.passes_per_step = b;
   }
   if (E->graph_ok) {
-    if (E->run_exec && !(same_run(R, E->run_key) && cs == E->key_cs && clusters == E->key_clusters))
-      drop_graph(E);
-    if (!E->run_exec) capture_run(E, R, cs, clusters);
+    if (E->run_exec && !(same_run(R, E->run_key) && E->launches == E->key_launches)) drop_graph(E);
+    if (!E->run_exec) capture_run(E, R);
   }
   // the events bracket the whole run: copies, queue reset and the launch
   ENS_CUDA(E, cudaEventRecord(E->ev[0], s));
   if (E->run_exec)
     ENS_CUDA(E, cudaGraphLaunch(E->run_exec, s));
   else
-    ENS_CUDA(E, enqueue_run(E, R, cs, clusters, s));
+    ENS_CUDA(E, enqueue_run(E, R, s));
   ENS_CUDA(E, cudaEventRecord(E->ev[1], s));
   ENS_CUDA(E, cudaStreamSynchronize(s));
   float t = 0.f;
@@ -367,8 +530,18 @@ erem_status run(erem_ens* E, int steps, cudaStream_t s) {
   erem_ens_run_stats& r = E->rs;
   std::memset(&r, 0, sizeof(r));
   r.t_ms = t;
-  r.cluster_ctas = cs;
-  r.clusters = clusters;
+  {  // the shape of the launch with the most work
+    double most = -1.0;
+    for (const EnsLaunch& L : E->launches) {
+      double sum = 0.0;
+      for (int k = 0; k < L.count; ++k) sum += member_weight(E, E->order_h[L.first + k]);
+      if (sum > most) {
+        most = sum;
+        r.cluster_ctas = L.cs;
+        r.clusters = L.clusters;
+      }
+    }
+  }
   r.cta_threads = ens_cta_threads();
   r.graph = E->run_exec ? 1 : 0;
   E->last.assign(E->st_h, E->st_h + E->n);
@@ -594,11 +767,13 @@ erem_status erem_ensemble_autotune(erem_ens* E, int probe_steps, void* stream) {
   const std::vector<int> levels0 = E->level_start;
   const std::vector<double> rates0 = E->pass_rate;
   const erem_ens_config keep = E->cfg;
+  const int tuned0 = E->tuned_cs;
   const bool keep_policy = keep.substep_policy == EREM_ENS_KEEP_SUBSTEPS;
   auto restore = [&](erem_status st) {
     E->cfg = keep;
     E->level_start = levels0;
     E->pass_rate = rates0;
+    E->tuned_cs = tuned0;
     copy_all(false);
     cudaStreamSynchronize(s);
     return st;
@@ -610,15 +785,12 @@ erem_status erem_ensemble_autotune(erem_ens* E, int probe_steps, void* stream) {
   const std::vector<int> learned = E->level_start;
   const std::vector<double> rates = E->pass_rate;
   if (copy_all(false) != EREM_OK) return restore(EREM_ECUDA);
-  const int cand[4] = {2, 4, 8, 16};
+  const int cand[5] = {0, 2, 4, 8, 16};   // 0: the planned launches
+  E->tuned_cs = 0;
   double best = 1e300;
-  int best_cs = 0;
+  int best_cs = -1;
   for (int cs : cand) {
-    int fit = 0;
-    if (ens_max_clusters(E->prec, cs, &fit) != cudaSuccess || fit < 1) {
-      cudaGetLastError();
-      continue;
-    }
+    if (cs && fit_clusters(E, cs, false) < 1) continue;
     E->cfg.cluster_ctas = cs;
     E->level_start = keep_policy ? learned : levels0;
     E->pass_rate = rates;
@@ -631,7 +803,7 @@ erem_status erem_ensemble_autotune(erem_ens* E, int probe_steps, void* stream) {
     if (copy_all(false) != EREM_OK) return restore(EREM_ECUDA);
   }
   ENS_CUDA(E, cudaStreamSynchronize(s));
-  if (best_cs == 0) return restore(efail(E, EREM_ECUDA, "no cluster size fits the device"));
+  if (best_cs < 0) return restore(efail(E, EREM_ECUDA, "no cluster size fits the device"));
   E->cfg = keep;
   E->tuned_cs = best_cs;
   E->level_start = keep_policy ? learned : levels0;

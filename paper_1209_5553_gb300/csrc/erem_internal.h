@@ -118,6 +118,7 @@ struct EnsMember {
   const double* dd;     // kEnsMaxLevels tables of mmax + 1 divided differences
   StopParams sp;        // tolerances, window, m_max (delta unused)
   double dt, cg;        // step, c / gamma
+  double rsqrt_n;       // 1 / sqrt(cells)
 };
 
 // Arguments of one run of the batched kernel.
@@ -449,6 +450,11 @@ void launch_bicg_iter(const erem_ctx* c, double sigma, cudaStream_t s);
 int ens_cta_threads();
 cudaError_t ens_max_clusters(int prec, int cs, int* n);
 cudaError_t launch_ens_cluster(const EnsRun& R, int prec, int cs, int clusters, cudaStream_t s);
+// ... for members that fit on their cluster's shared memory
+bool ens_res_fits(int prec, int cs, int ny, int px, bool nd, int smem_optin);
+cudaError_t ens_res_max_clusters(int prec, int cs, int smem_optin, int* n);
+cudaError_t launch_ens_resident(const EnsRun& R, int prec, int cs, int clusters, int smem_optin,
+                                cudaStream_t s);
 void launch_unpack(const erem_ctx* c, const double* src, double* dst, cudaStream_t s);
 
 // Krylov (Arnoldi, modified Gram-Schmidt) passes, FP64
