@@ -158,6 +158,7 @@ PcPoly pc_poly(int deg, double lo = -1.0) {
 erem_status ensure_mg(erem_ctx* c) {
   if (!c->pc_diag) EREM_TRY(dalloc_t(c, &c->pc_diag, (size_t)c->Np));
   if (!c->mg.empty()) return EREM_OK;
+  c->mg_small = mg_small_fits(c);
   int nx = c->nx, ny = c->ny, nz = c->nz;
   while (c->mg.empty() || (long long)nx * ny * nz > kMgCoarsest) {
     const int cx = (nx + 1) / 2, cy = (ny + 1) / 2, cz = c->dim == 3 ? (nz + 1) / 2 : 1;
@@ -963,6 +964,7 @@ void fill_interval(const erem_ctx* c, erem_stats* st) {
 // > 1 until at most kMgCoarsest cells remain (at least one coarse level).
 erem_status ensure_smg(erem_ctx* c) {
   if (!c->smg.empty()) return EREM_OK;
+  c->mg_small = mg_small_fits(c);
   int nx = c->nx, ny = c->ny, nz = c->nz;
   const int nk = c->dim == 3 ? 6 : 4;
   auto add = [&](int ax, int ay, int az, size_t n) -> erem_status {

@@ -238,6 +238,7 @@ struct erem_ctx {
   // and the coarse levels 1..L (levels[0] is the first coarse level)
   float* pc_diag = nullptr;
   std::vector<erem::MgLevel> mg;
+  bool mg_small = false;      // the device runs the small levels of a V-cycle in one launch
   int mg_nu = 3;          // Chebyshev-Jacobi smoothing steps before and after
   float mg_omega = 1.8f;  // weight of the coarse correction
   // two preconditioned CG iterations (even, odd) captured as one CUDA graph,
@@ -434,6 +435,7 @@ void launch_pc_setup(const erem_ctx* c, cudaStream_t s);
 // `poly` as its smoother when pc_deg = 0); returns the buffer that holds z.
 const float* launch_pc_apply(const erem_ctx* c, const PcPoly& poly, cudaStream_t s);
 void launch_pcg_iter(const erem_ctx* c, const PcPoly& poly, const float* z, int k, cudaStream_t s);
+bool mg_small_fits(const erem_ctx* c);
 void launch_mg_setup(const erem_ctx* c, cudaStream_t s);
 // stage multigrid: operators of every level for sigma I - J; one BiCGSTAB
 // iteration with the V-cycle as right preconditioner

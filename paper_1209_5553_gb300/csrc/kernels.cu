@@ -11,6 +11,7 @@
 // the last block to finish (atomic ticket) sums the partials in block order
 // and writes the result into the control block.  Min/max reductions are
 // exact in any order.
+#include <cstdlib>
 #include <algorithm>
 #include <cstdint>
 
@@ -2063,6 +2064,24 @@ __device__ __forceinline__ float mg_offdiag(const MgL& L, const float* __restric
   return s;
 }
 
+// (N x)_i with x a function of the cell index and its coordinates
+template <typename F>
+__device__ __forceinline__ float mg_offdiag_of(const MgL& L, F&& x, int ip, int ix, int iy, int iz) {
+  float s = 0.0f;
+  if (ix < L.g.nx - 1) s = fmaf(L.Ux[ip], x(ip + 1, ix + 1, iy, iz), s);
+  if (ix > 0) s = fmaf(L.Ux[ip - 1], x(ip - 1, ix - 1, iy, iz), s);
+  if (iy < L.g.ny - 1) s = fmaf(L.Uy[ip], x(ip + L.g.px, ix, iy + 1, iz), s);
+  if (iy > 0) s = fmaf(L.Uy[ip - L.g.px], x(ip - L.g.px, ix, iy - 1, iz), s);
+  if (L.g.dim == 3) {
+    if (iz < L.g.nz - 1) s = fmaf(L.Uz[ip], x(ip + L.g.plane, ix, iy, iz + 1), s);
+    if (iz > 0) s = fmaf(L.Uz[ip - L.g.plane], x(ip - L.g.plane, ix, iy, iz - 1), s);
+  }
+  return s;
+}
+__device__ __forceinline__ float mg_cheb(float z, float zp, float c1, float c2, float dinv, float s) {
+  return fmaf(c2, fmaf(dinv, s, -z), fmaf(c1, z - zp, z));
+}
+
 // One Chebyshev-Jacobi step on a coarse level: xn = xc + c1 (xc - xp) +
 // c2 (D^-1 (rhs + N xc) - xc); xc = NULL means x = 0 (xn = c2 D^-1 rhs),
 // xp = NULL means 0.
@@ -2080,6 +2099,40 @@ __global__ void k_mg_sweep(MgL L, const float* __restrict__ rhs, const float* __
     const float zp = xp ? xp[ip] : 0.0f;
     const float s = rhs[ip] + mg_offdiag(L, xc, ip, ix, iy, iz);
     xn[ip] = z + c1 * (z - zp) + c2 * fmaf(L.dinv[ip], s, -z);
+  }
+}
+
+// The first two Chebyshev-Jacobi steps from zero in one pass (the first formed
+// where the second reads it), with the same values and order of sums; the first
+// one's vector goes to xf if a third step needs it (may be null).
+__global__ void k_mg_sweep2(MgL L, const float* __restrict__ rhs, float* __restrict__ xf,
+                            float* __restrict__ xn, float b0, float c1, float c2) {
+  auto first = [&](int j, int, int, int) { return b0 * (L.dinv[j] * rhs[j]); };
+  for (int i = blockIdx.x * NT + threadIdx.x; i < L.g.N; i += gridDim.x * NT) {
+    int ix, iy, iz, ip;
+    cell_of(i, L.g, ix, iy, iz, ip);
+    const float z = first(ip, ix, iy, iz);
+    xn[ip] = mg_cheb(z, 0.0f, c1, c2, L.dinv[ip], rhs[ip] + mg_offdiag_of(L, first, ip, ix, iy, iz));
+    if (xf) xf[ip] = z;
+  }
+}
+
+// x_f + omega P x_c and one Chebyshev-Jacobi step from it in one pass; the
+// corrected vector goes to xp (the next step's vector before the last; may be
+// null).
+__global__ void k_mg_prolong_sweep(MgL L, const float* __restrict__ rhs, const float* __restrict__ x_f,
+                                   Geo cg, const float* __restrict__ x_c, float omega,
+                                   float* __restrict__ xp, float* __restrict__ xn, float c1, float c2) {
+  auto corrected = [&](int q, int ix, int iy, int iz) {
+    const int I = (ix >> 1) + cg.px * ((iy >> 1) + cg.ny * (L.g.dim == 3 ? (iz >> 1) : 0));
+    return fmaf(omega, x_c[I], x_f[q]);
+  };
+  for (int i = blockIdx.x * NT + threadIdx.x; i < L.g.N; i += gridDim.x * NT) {
+    int ix, iy, iz, ip;
+    cell_of(i, L.g, ix, iy, iz, ip);
+    const float z = corrected(ip, ix, iy, iz);
+    xn[ip] = mg_cheb(z, 0.0f, c1, c2, L.dinv[ip], rhs[ip] + mg_offdiag_of(L, corrected, ip, ix, iy, iz));
+    if (xp) xp[ip] = z;
   }
 }
 
@@ -2305,6 +2358,255 @@ k_mg_coarse_apply(const float* __restrict__ inv, const float* __restrict__ b, fl
   }
   for (; j < N; ++j) a0 = fmaf(inv[(size_t)j * N + i], bs[j], a0);
   x[i] = (a0 + a1) + (a2 + a3);
+}
+
+// ---------------------------------------------------------------------------
+// The small levels of a V-cycle in one launch.  From about 4000 cells down a
+// sweep is far shorter than the launch that starts it (2 us in a replayed
+// graph, eight to a level), and a level's operator and vectors fit in the
+// shared memory of one SM: CTA 0 of a cluster loads them and runs the levels
+// with a block barrier between operations.  For the coarsest solve every CTA
+// of the cluster holds a slice of the rows of the inverse (loaded while CTA 0
+// is on the way down), takes the right-hand side from CTA 0's shared memory and
+// writes its part of the correction back.  The first sweep from zero and the
+// prolongation are formed where the next sweep reads them.  Every value has the
+// bits of the single launches.  Pressure at 128^3: 25 us, where the product with
+// the coarsest inverse alone took 37.6; stage systems at 512^2 (64^2, 32^2 and
+// 16^2, one CTA): 19.6 us, half of it in loading the operators and in the 40
+// sweeps of the coarsest level.
+// ---------------------------------------------------------------------------
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallCtas = 16;
+constexpr int kSmallLevels = 8;
+
+// The cells' coordinates, packed into 16 bits each (a small level has at most
+// 2^12 cells or so; the bits of its three dimensions add up to at most 15): a
+// single SM runs these levels, and two integer divisions per cell and operation
+// would be most of its instructions.
+struct SmallCell {
+  const unsigned short* co;
+  int bx, by;   // bits of ix and iy
+  __device__ __forceinline__ void operator()(int i, int& ix, int& iy, int& iz) const {
+    const int v = co[i];
+    ix = v & ((1 << bx) - 1);
+    iy = (v >> bx) & ((1 << by) - 1);
+    iz = v >> (bx + by);
+  }
+};
+__host__ __device__ inline int bits_of(int n) {   // of 0 .. n - 1
+  int b = 0;
+  while ((1 << b) < n) ++b;
+  return b;
+}
+// floats that hold the coordinates of n cells
+__host__ __device__ inline int coord_floats(int n) { return (n + 1) / 2; }
+__device__ __forceinline__ SmallCell fill_cells(const Geo& g, float* at, int tid, int threads) {
+  SmallCell c;
+  c.bx = bits_of(g.nx);
+  c.by = bits_of(g.ny);
+  unsigned short* co = reinterpret_cast<unsigned short*>(at);
+  c.co = co;
+  for (int i = tid; i < g.N; i += threads) {
+    int ix, iy, iz, ip;
+    cell_of(i, g, ix, iy, iz, ip);
+    co[i] = (unsigned short)(ix | (iy << c.bx) | (iz << (c.bx + c.by)));
+  }
+  return c;
+}
+
+struct MgSmall {
+  MgL L[kSmallLevels];         // the levels, finest first
+  int off[kSmallLevels];       // their arrays in shared memory (floats): dinv diag Ux Uy Uz rhs x0 x1 coordinates
+  int n;
+  const float* rhs;            // of the finest
+  float* x;                    // its correction
+  const float* inv;            // of the coarsest operator, by columns
+  int inv_off, inv_stride;     // this CTA's rows of it in shared memory
+  int nu;
+  float c1[16], c2[16], omega;
+  const Ctrl* ctrl;
+};
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ unsigned map_cta0(const void* p) {
+  unsigned r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(p)));
+  return r;
+}
+__device__ __forceinline__ float ld_cluster(unsigned p) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_cluster(unsigned p, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(p), "f"(v) : "memory");
+}
+
+__global__ void __launch_bounds__(kSmallThreads, 1) k_mg_small(const __grid_constant__ MgSmall A) {
+  extern __shared__ __align__(16) float sm[];
+  if (*(volatile const int*)&A.ctrl->lin_done) return;   // the same value in every CTA
+  const int rank = blockIdx.x, tid = threadIdx.x;
+  const int NC = A.L[A.n - 1].g.N;
+  const int per = (NC + kSmallCtas - 1) / kSmallCtas;      // rows of the inverse per CTA
+  const int i0 = min(rank * per, NC), i1 = min(i0 + per, NC);
+  float* const inv = sm + A.inv_off;
+  // the arrays of level l in shared memory
+  auto level = [&](int l, float*& rhs, float*& xa, float*& xb) {
+    MgL S = A.L[l];
+    const int N = S.g.N, nu = S.g.dim == 3 ? 3 : 2;
+    float* p = sm + A.off[l];
+    S.dinv = p;
+    S.diag = p + N;
+    S.Ux = p + 2 * N;
+    S.Uy = p + 3 * N;
+    S.Uz = p + 4 * N;
+    rhs = p + (2 + nu) * N;
+    xa = rhs + N;
+    xb = xa + N;
+    return S;
+  };
+  auto cells = [&](int l) {
+    const Geo& g = A.L[l].g;
+    SmallCell c;
+    c.co = reinterpret_cast<const unsigned short*>(sm + A.off[l] + (g.dim == 3 ? 8 : 7) * g.N);
+    c.bx = bits_of(g.nx);
+    c.by = bits_of(g.ny);
+    return c;
+  };
+  if (rank == 0) {
+    for (int l = 0; l < A.n; ++l) {
+      float *rhs, *xa, *xb;
+      const MgL S = level(l, rhs, xa, xb);
+      const MgL& G = A.L[l];
+      if (l + 1 < A.n)
+        for (int i = tid; i < G.g.N; i += kSmallThreads) {
+          S.dinv[i] = G.dinv[i];
+          S.diag[i] = G.diag[i];
+          S.Ux[i] = G.Ux[i];
+          S.Uy[i] = G.Uy[i];
+          if (G.g.dim == 3) S.Uz[i] = G.Uz[i];
+        }
+      if (l == 0)
+        for (int i = tid; i < G.g.N; i += kSmallThreads) rhs[i] = A.rhs[i];
+      fill_cells(G.g, sm + A.off[l] + (G.g.dim == 3 ? 8 : 7) * G.g.N, tid, kSmallThreads);
+    }
+  }
+  for (int k = tid; k < NC * (i1 - i0); k += kSmallThreads) {
+    const int j = k / (i1 - i0), i = k - j * (i1 - i0);
+    inv[j * A.inv_stride + i] = A.inv[(size_t)j * NC + i0 + i];
+  }
+  __syncthreads();
+  float *brhs, *bx, *bt;   // the coarsest level's
+  level(A.n - 1, brhs, bx, bt);
+  if (rank == 0) {
+    for (int l = 0; l + 1 < A.n; ++l) {
+      float *rhs, *xc, *xo;
+      const MgL S = level(l, rhs, xc, xo);
+      const SmallCell at = cells(l), cat = cells(l + 1);
+      auto first = [&](int j, int, int, int) { return A.c2[0] * (S.dinv[j] * rhs[j]); };
+      if (A.nu == 1) {
+        for (int i = tid; i < S.g.N; i += kSmallThreads) xc[i] = first(i, 0, 0, 0);
+        __syncthreads();
+      }
+      // sweep j writes over the vector before the last, read at its own cell only
+      for (int j = 1; j < A.nu; ++j) {
+        for (int i = tid; i < S.g.N; i += kSmallThreads) {
+          const int ip = i;
+          int ix, iy, iz;
+          at(i, ix, iy, iz);
+          auto cur = [&](int q, int, int, int) { return xc[q]; };
+          const float z = j == 1 ? first(ip, ix, iy, iz) : xc[ip];
+          const float zp = j == 1 ? 0.0f : j == 2 ? first(ip, ix, iy, iz) : xo[ip];
+          const float s = rhs[ip] + (j == 1 ? mg_offdiag_of(S, first, ip, ix, iy, iz)
+                                            : mg_offdiag_of(S, cur, ip, ix, iy, iz));
+          xo[ip] = mg_cheb(z, zp, A.c1[j], A.c2[j], S.dinv[ip], s);
+        }
+        __syncthreads();
+        float* t = xo;
+        xo = xc;
+        xc = t;
+      }
+      float *crhs, *ca, *cb;
+      const MgL C = level(l + 1, crhs, ca, cb);
+      for (int I = tid; I < C.g.N; I += kSmallThreads) {
+        int X, Y, Z;
+        cat(I, X, Y, Z);
+        const int xe = min(2 * X + 2, S.g.nx), ye = min(2 * Y + 2, S.g.ny);
+        const int ze = S.g.dim == 3 ? min(2 * Z + 2, S.g.nz) : 1;
+        auto cur = [&](int q, int, int, int) { return xc[q]; };
+        float acc = 0.0f;
+        for (int iz = (S.g.dim == 3 ? 2 * Z : 0); iz < ze; ++iz)
+          for (int iy = 2 * Y; iy < ye; ++iy)
+            for (int ix = 2 * X; ix < xe; ++ix) {
+              const int ip = ix + S.g.px * (iy + S.g.ny * iz);
+              acc += rhs[ip] - fmaf(S.diag[ip], xc[ip], -mg_offdiag_of(S, cur, ip, ix, iy, iz));
+            }
+        crhs[I] = acc;
+      }
+      __syncthreads();
+    }
+  }
+  cluster_sync();
+  {
+    // x = inv b: four chains per row (k_mg_coarse_apply's), one thread each
+    float* const b = inv + NC * A.inv_stride;
+    const unsigned b0 = map_cta0(brhs), x0 = map_cta0(bx);
+    for (int j = tid; j < NC; j += kSmallThreads) b[j] = ld_cluster(b0 + 4u * j);
+    __syncthreads();
+    for (int k = tid; k < (per + 7) / 8 * 32; k += kSmallThreads) {   // whole warps
+      const int r = k >> 2, q = k & 3;
+      float a = 0.0f;
+      if (r < i1 - i0) {
+        int j = 0;
+        for (; j + 4 <= NC; j += 4) a = fmaf(inv[(j + q) * A.inv_stride + r], b[j + q], a);
+        if (q == 0)
+          for (; j < NC; ++j) a = fmaf(inv[j * A.inv_stride + r], b[j], a);
+      }
+      a += __shfl_xor_sync(0xffffffffu, a, 1);
+      a += __shfl_xor_sync(0xffffffffu, a, 2);
+      if (q == 0 && r < i1 - i0) st_cluster(x0 + 4u * (i0 + r), a);
+    }
+  }
+  cluster_sync();
+  if (rank != 0) return;
+  const float* xcoarse = bx;
+  for (int l = A.n - 2; l >= 0; --l) {
+    float *rhs, *xa, *xb;
+    const MgL S = level(l, rhs, xa, xb);
+    const SmallCell at = cells(l);
+    const Geo& cg = A.L[l + 1].g;
+    // the way down left its result in xa after an even number of swaps
+    float* xc = (A.nu - 1) & 1 ? xb : xa;
+    float* xo = (A.nu - 1) & 1 ? xa : xb;
+    const float* xd = xc;
+    auto corrected = [&](int q, int ix, int iy, int iz) {
+      const int I = (ix >> 1) + cg.px * ((iy >> 1) + cg.ny * (S.g.dim == 3 ? (iz >> 1) : 0));
+      return fmaf(A.omega, xcoarse[I], xd[q]);
+    };
+    for (int j = 0; j < A.nu; ++j) {
+      // sweep 1 needs the corrected vector once more at its own cell and writes
+      // over it; from sweep 2 on as on the way down
+      for (int i = tid; i < S.g.N; i += kSmallThreads) {
+        const int ip = i;
+        int ix, iy, iz;
+        at(i, ix, iy, iz);
+        auto cur = [&](int q, int, int, int) { return xc[q]; };
+        const float z = j == 0 ? corrected(ip, ix, iy, iz) : xc[ip];
+        const float zp = j == 0 ? 0.0f : j == 1 ? corrected(ip, ix, iy, iz) : xo[ip];
+        const float s = rhs[ip] + (j == 0 ? mg_offdiag_of(S, corrected, ip, ix, iy, iz)
+                                          : mg_offdiag_of(S, cur, ip, ix, iy, iz));
+        xo[ip] = mg_cheb(z, zp, A.c1[j], A.c2[j], S.dinv[ip], s);
+      }
+      __syncthreads();
+      float* t = xo;
+      xo = xc;
+      xc = t;
+    }
+    xcoarse = xc;
+  }
+  for (int i = tid; i < A.L[0].g.N; i += kSmallThreads) A.x[i] = xcoarse[i];
 }
 
 // x += alpha d, r -= alpha Ad; rr -> convergence (the preconditioner's
@@ -2625,6 +2927,20 @@ __device__ __forceinline__ float smg_offdiag(const MgN& L, const float* __restri
   return s;
 }
 
+template <typename F>
+__device__ __forceinline__ float smg_offdiag_of(const MgN& L, F&& x, int ip, int ix, int iy, int iz) {
+  float s = 0.0f;
+  if (ix > 0) s = fmaf(L.c[0][ip], x(ip - 1, ix - 1, iy, iz), s);
+  if (ix < L.g.nx - 1) s = fmaf(L.c[1][ip], x(ip + 1, ix + 1, iy, iz), s);
+  if (iy > 0) s = fmaf(L.c[2][ip], x(ip - L.g.px, ix, iy - 1, iz), s);
+  if (iy < L.g.ny - 1) s = fmaf(L.c[3][ip], x(ip + L.g.px, ix, iy + 1, iz), s);
+  if (L.g.dim == 3) {
+    if (iz > 0) s = fmaf(L.c[4][ip], x(ip - L.g.plane, ix, iy, iz - 1), s);
+    if (iz < L.g.nz - 1) s = fmaf(L.c[5][ip], x(ip + L.g.plane, ix, iy, iz + 1), s);
+  }
+  return s;
+}
+
 // level 0: D = sigma - J_ii, c_k = J's coupling k (J >= 0 off the diagonal)
 __global__ void k_smg_setup(JIn J, double sigma, MgN L) {
   for (int i = blockIdx.x * NT + threadIdx.x; i < L.g.N; i += gridDim.x * NT) {
@@ -2669,18 +2985,46 @@ __global__ void k_smg_coarsen(MgN f, MgN c) {
   }
 }
 
-// damped Jacobi: xo = xi + w D^-1 (rhs - A xi); xi = NULL means 0
+// damped Jacobi: xo = xi + w D^-1 (rhs - A xi)
 __global__ void k_smg_jacobi(MgN L, const float* __restrict__ rhs, const float* __restrict__ xi,
                              float* __restrict__ xo, float w) {
   for (int i = blockIdx.x * NT + threadIdx.x; i < L.g.N; i += gridDim.x * NT) {
     int ix, iy, iz, ip;
     cell_of(i, L.g, ix, iy, iz, ip);
-    if (!xi) {
-      xo[ip] = w * L.Dinv[ip] * rhs[ip];
-      continue;
-    }
     const float x = xi[ip];
     const float res = rhs[ip] - fmaf(L.D[ip], x, -smg_offdiag(L, xi, ip, ix, iy, iz));
+    xo[ip] = fmaf(w * L.Dinv[ip], res, x);
+  }
+}
+
+// The first two damped Jacobi sweeps from zero in one pass (the first formed
+// where the second reads it).  These levels are launch-bound (1.7 us a sweep at
+// 512^2 and below): four launches of a level in place of six, and the same
+// values and order of sums as sweep by sweep.  A V-cycle at 512^2, with the small
+// levels in k_smg_small: 59 -> 46 us.
+__global__ void k_smg_jacobi2(MgN L, const float* __restrict__ rhs, float* __restrict__ xo, float w) {
+  auto first = [&](int j, int, int, int) { return w * L.Dinv[j] * rhs[j]; };
+  for (int i = blockIdx.x * NT + threadIdx.x; i < L.g.N; i += gridDim.x * NT) {
+    int ix, iy, iz, ip;
+    cell_of(i, L.g, ix, iy, iz, ip);
+    const float x = first(ip, ix, iy, iz);
+    const float res = rhs[ip] - fmaf(L.D[ip], x, -smg_offdiag_of(L, first, ip, ix, iy, iz));
+    xo[ip] = fmaf(w * L.Dinv[ip], res, x);
+  }
+}
+
+// x_f + P x_c and one damped Jacobi sweep from it in one pass.
+__global__ void k_smg_prolong_jacobi(MgN L, const float* __restrict__ rhs, const float* __restrict__ x_f,
+                                     Geo cg, const float* __restrict__ x_c, float* __restrict__ xo,
+                                     float w) {
+  auto corrected = [&](int q, int ix, int iy, int iz) {
+    return x_f[q] + x_c[(ix >> 1) + cg.px * ((iy >> 1) + cg.ny * (L.g.dim == 3 ? (iz >> 1) : 0))];
+  };
+  for (int i = blockIdx.x * NT + threadIdx.x; i < L.g.N; i += gridDim.x * NT) {
+    int ix, iy, iz, ip;
+    cell_of(i, L.g, ix, iy, iz, ip);
+    const float x = corrected(ip, ix, iy, iz);
+    const float res = rhs[ip] - fmaf(L.D[ip], x, -smg_offdiag_of(L, corrected, ip, ix, iy, iz));
     xo[ip] = fmaf(w * L.Dinv[ip], res, x);
   }
 }
@@ -2701,15 +3045,6 @@ __global__ void k_smg_restrict(MgN f, const float* __restrict__ rhs_f, const flo
           acc += rhs_f[ip] - fmaf(f.D[ip], x_f[ip], -smg_offdiag(f, x_f, ip, ix, iy, iz));
         }
     rhs_c[IP] = acc;
-  }
-}
-
-// x_f += P x_c
-__global__ void k_smg_prolong(Geo fg, float* __restrict__ x_f, Geo cg, const float* __restrict__ x_c) {
-  for (int i = blockIdx.x * NT + threadIdx.x; i < fg.N; i += gridDim.x * NT) {
-    int ix, iy, iz, ip;
-    cell_of(i, fg, ix, iy, iz, ip);
-    x_f[ip] += x_c[(ix >> 1) + cg.px * ((iy >> 1) + cg.ny * (fg.dim == 3 ? (iz >> 1) : 0))];
   }
 }
 
@@ -2741,12 +3076,12 @@ __global__ void __launch_bounds__(512) k_smg_coarse(MgN L, const float* __restri
 }
 
 // Coarsest level with at most 512 cells: the damped Jacobi sweeps of
-// k_smg_coarse with one cell per thread, its coefficients and rhs in registers
-// and the iterate in shared memory (two buffers, one block sync per sweep).
-__global__ void __launch_bounds__(512) k_smg_coarse1(MgN L, const float* __restrict__ rhs,
-                                                     float* __restrict__ x, int sweeps, float w) {
-  __shared__ float xs[2][512];
-  const int N = L.g.N;
+// k_smg_coarse with one cell per thread of one CTA, its coefficients and rhs in
+// registers and the iterate in shared memory (two buffers, one block sync per
+// sweep).
+__device__ void smg_coarse_block(const MgN& L, const float* rhs, float* x, int sweeps, float w,
+                                 float (*xs)[512]) {
+  const int N = L.g.N, threads = (N + 31) / 32 * 32;
   const bool own = (int)threadIdx.x < N;
   int ix = 0, iy = 0, iz = 0, ip = 0;
   float d = 0.0f, wdi = 0.0f, r = 0.0f, cw = 0.0f, ce = 0.0f, cs = 0.0f, cn = 0.0f, cb = 0.0f,
@@ -2769,7 +3104,8 @@ __global__ void __launch_bounds__(512) k_smg_coarse1(MgN L, const float* __restr
   }
   int cur = 0;
   for (int it = 1; it < sweeps; ++it) {
-    __syncthreads();  // xs[cur] complete
+    // xs[cur] complete: the warps that own cells
+    asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
     if (own) {
       const float* a = xs[cur];
       float o = 0.0f;
@@ -2788,6 +3124,143 @@ __global__ void __launch_bounds__(512) k_smg_coarse1(MgN L, const float* __restr
     cur ^= 1;
   }
   if (own) x[ip] = xv;
+}
+
+__global__ void __launch_bounds__(512) k_smg_coarse1(MgN L, const float* __restrict__ rhs,
+                                                     float* __restrict__ x, int sweeps, float w) {
+  __shared__ float xs[2][512];
+  if ((int)threadIdx.x < (L.g.N + 31) / 32 * 32) smg_coarse_block(L, rhs, x, sweeps, w, xs);
+}
+
+// The small levels of one V-cycle of the stage systems in one CTA, operators
+// and vectors in shared memory (see k_mg_small): two damped Jacobi sweeps down
+// (the first from zero, formed where the second reads it), the restriction,
+// the coarsest sweeps, two sweeps up (the prolongation formed where the first
+// of them reads it).
+struct SmgSmall {
+  MgN L[kSmallLevels];
+  int off[kSmallLevels];   // D Dinv c[0..] rhs x0 x1
+  int n;
+  const float* rhs;
+  float* x;
+  int sweeps;
+  float w;
+  const Ctrl* ctrl;
+};
+
+__global__ void __launch_bounds__(kSmallThreads, 1) k_smg_small(const __grid_constant__ SmgSmall A) {
+  extern __shared__ __align__(16) float sm[];
+  __shared__ float xs[2][512];
+  if (*(volatile const int*)&A.ctrl->lin_done) return;
+  const int tid = threadIdx.x;
+  const float w = A.w;
+  auto level = [&](int l, float*& rhs, float*& xa, float*& xb) {
+    MgN S = A.L[l];
+    const int N = S.g.N, nk = S.g.dim == 3 ? 6 : 4;
+    float* p = sm + A.off[l];
+    S.D = p;
+    S.Dinv = p + N;
+    for (int k = 0; k < 6; ++k) S.c[k] = p + (2 + (k < nk ? k : 0)) * N;
+    rhs = p + (2 + nk) * N;
+    xa = rhs + N;
+    xb = xa + N;
+    return S;
+  };
+  auto cells = [&](int l) {
+    const Geo& g = A.L[l].g;
+    SmallCell c;
+    c.co = reinterpret_cast<const unsigned short*>(sm + A.off[l] + (g.dim == 3 ? 11 : 9) * g.N);
+    c.bx = bits_of(g.nx);
+    c.by = bits_of(g.ny);
+    return c;
+  };
+  for (int l = 0; l < A.n; ++l) {
+    float *rhs, *xa, *xb;
+    const MgN S = level(l, rhs, xa, xb);
+    const MgN& G = A.L[l];
+    const int nk = G.g.dim == 3 ? 6 : 4;
+    for (int i = tid; i < G.g.N; i += kSmallThreads) {
+      S.D[i] = G.D[i];
+      S.Dinv[i] = G.Dinv[i];
+#pragma unroll
+      for (int k = 0; k < 6; ++k)
+        if (k < nk) S.c[k][i] = G.c[k][i];
+      if (l == 0) rhs[i] = A.rhs[i];
+    }
+    fill_cells(G.g, sm + A.off[l] + (G.g.dim == 3 ? 11 : 9) * G.g.N, tid, kSmallThreads);
+  }
+  __syncthreads();
+  for (int l = 0; l + 1 < A.n; ++l) {
+    float *rhs, *xa, *xb;
+    const MgN S = level(l, rhs, xa, xb);
+    const SmallCell at = cells(l), cat = cells(l + 1);
+    auto first = [&](int j, int, int, int) { return w * S.Dinv[j] * rhs[j]; };
+    for (int i = tid; i < S.g.N; i += kSmallThreads) {
+      const int ip = i;
+      int ix, iy, iz;
+      at(i, ix, iy, iz);
+      const float x = first(ip, ix, iy, iz);
+      const float res = rhs[ip] - fmaf(S.D[ip], x, -smg_offdiag_of(S, first, ip, ix, iy, iz));
+      xb[ip] = fmaf(w * S.Dinv[ip], res, x);
+    }
+    __syncthreads();
+    float *crhs, *ca, *cb;
+    const MgN C = level(l + 1, crhs, ca, cb);
+    auto cur = [&](int q, int, int, int) { return xb[q]; };
+    for (int I = tid; I < C.g.N; I += kSmallThreads) {
+      int X, Y, Z;
+      cat(I, X, Y, Z);
+      const int xe = min(2 * X + 2, S.g.nx), ye = min(2 * Y + 2, S.g.ny);
+      const int ze = S.g.dim == 3 ? min(2 * Z + 2, S.g.nz) : 1;
+      float acc = 0.0f;
+      for (int iz = (S.g.dim == 3 ? 2 * Z : 0); iz < ze; ++iz)
+        for (int iy = 2 * Y; iy < ye; ++iy)
+          for (int ix = 2 * X; ix < xe; ++ix) {
+            const int ip = ix + S.g.px * (iy + S.g.ny * iz);
+            acc += rhs[ip] - fmaf(S.D[ip], xb[ip], -smg_offdiag_of(S, cur, ip, ix, iy, iz));
+          }
+      crhs[I] = acc;
+    }
+    __syncthreads();
+  }
+  const float* xcoarse;
+  {
+    float *rhs, *xa, *xb;
+    const MgN S = level(A.n - 1, rhs, xa, xb);
+    if (tid < (S.g.N + 31) / 32 * 32) smg_coarse_block(S, rhs, xa, A.sweeps, w, xs);
+    xcoarse = xa;
+    __syncthreads();
+  }
+  for (int l = A.n - 2; l >= 0; --l) {
+    float *rhs, *xa, *xb;
+    const MgN S = level(l, rhs, xa, xb);
+    const Geo& cg = A.L[l + 1].g;
+    const SmallCell at = cells(l);
+    auto corrected = [&](int q, int ix, int iy, int iz) {
+      return xb[q] + xcoarse[(ix >> 1) + cg.px * ((iy >> 1) + cg.ny * (S.g.dim == 3 ? (iz >> 1) : 0))];
+    };
+    for (int i = tid; i < S.g.N; i += kSmallThreads) {
+      const int ip = i;
+      int ix, iy, iz;
+      at(i, ix, iy, iz);
+      const float x = corrected(ip, ix, iy, iz);
+      const float res = rhs[ip] - fmaf(S.D[ip], x, -smg_offdiag_of(S, corrected, ip, ix, iy, iz));
+      xa[ip] = fmaf(w * S.Dinv[ip], res, x);
+    }
+    __syncthreads();
+    auto cur = [&](int q, int, int, int) { return xa[q]; };
+    for (int i = tid; i < S.g.N; i += kSmallThreads) {
+      const int ip = i;
+      int ix, iy, iz;
+      at(i, ix, iy, iz);
+      const float x = xa[ip];
+      const float res = rhs[ip] - fmaf(S.D[ip], x, -smg_offdiag_of(S, cur, ip, ix, iy, iz));
+      xb[ip] = fmaf(w * S.Dinv[ip], res, x);
+    }
+    __syncthreads();
+    xcoarse = xb;
+  }
+  for (int i = tid; i < A.L[0].g.N; i += kSmallThreads) A.x[i] = xcoarse[i];
 }
 
 // BiCGSTAB with the V-cycle as right preconditioner: the direction and the
@@ -3298,6 +3771,35 @@ MgL mg_level(const erem_ctx* c, int l) {
 }
 }  // namespace
 
+// Whether the device runs the small levels' launches (a cluster of 16 CTAs with
+// most of an SM's shared memory each).
+bool mg_small_fits(const erem_ctx* c) {
+  if (const char* e = std::getenv("EREM_MG_SMALL"))  // tuning override: 0 launches every level
+    if (std::atoi(e) == 0) return false;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kSmallCtas);
+  cfg.blockDim = dim3(kSmallThreads);
+  cfg.dynamicSmemBytes = (size_t)c->smem_optin - 6144;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = kSmallCtas;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  const void *a = (const void*)k_mg_small, *b = (const void*)k_smg_small;
+  if (c->smem_optin < 65536 ||
+      cudaFuncSetAttribute(a, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+      cudaFuncSetAttribute(a, cudaFuncAttributeMaxDynamicSharedMemorySize, c->smem_optin - 1024) != cudaSuccess ||
+      cudaFuncSetAttribute(b, cudaFuncAttributeMaxDynamicSharedMemorySize, c->smem_optin - 6144) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, a, &cfg) != cudaSuccess || n < 1) {
+    cudaGetLastError();
+    return false;
+  }
+  return true;
+}
+
 // Galerkin operators of the coarse levels, after launch_pc_setup, and the
 // inverse of the coarsest one.
 void launch_mg_setup(const erem_ctx* c, cudaStream_t s) {
@@ -3316,23 +3818,91 @@ void launch_mg_setup(const erem_ctx* c, cudaStream_t s) {
 }
 
 namespace {
-// smoothing on coarse level l: deg Chebyshev-Jacobi steps from x = 0 (pre) or
-// from x[*cur] (post); returns the buffer index holding the result
-int mg_smooth(const erem_ctx* c, int l, const PcPoly& poly, int cur, bool from_zero, cudaStream_t s) {
+// smoothing on coarse level l: deg Chebyshev-Jacobi steps from x = 0; returns
+// the buffer index holding the result
+int mg_presmooth(const erem_ctx* c, int l, const PcPoly& poly, cudaStream_t s) {
   const MgL L = mg_level(c, l);
   const MgLevel& m = c->mg[l];
   const int nb = grid_for(c, L.g.N);
-  int prev = -1;
-  for (int j = 0; j < poly.deg; ++j) {
-    const int nxt = from_zero && j == 0 ? 0 : (cur + 1) % 3;
-    const float* xc = (from_zero && j == 0) ? nullptr : m.x[cur];
-    const float* xp = prev >= 0 ? m.x[prev] : nullptr;
+  if (poly.deg == 1) {
     ++c->launches;
-    k_mg_sweep<<<nb, NT, 0, s>>>(L, m.rhs, xp, xc, m.x[nxt], (float)poly.c1[j], (float)poly.c2[j]);
-    prev = (from_zero && j == 0) ? -1 : cur;
+    k_mg_sweep<<<nb, NT, 0, s>>>(L, m.rhs, nullptr, nullptr, m.x[0], (float)poly.c1[0], (float)poly.c2[0]);
+    return 0;
+  }
+  ++c->launches;
+  k_mg_sweep2<<<nb, NT, 0, s>>>(L, m.rhs, poly.deg > 2 ? m.x[0] : nullptr, m.x[1], (float)poly.c2[0], (float)poly.c1[1], (float)poly.c2[1]);
+  int cur = 1;
+  for (int j = 2; j < poly.deg; ++j) {
+    const int nxt = (cur + 1) % 3;
+    ++c->launches;
+    k_mg_sweep<<<nb, NT, 0, s>>>(L, m.rhs, m.x[(cur + 2) % 3], m.x[cur], m.x[nxt], (float)poly.c1[j],
+                                 (float)poly.c2[j]);
     cur = nxt;
   }
   return cur;
+}
+
+// ... the correction x_c of the level below and deg steps from x[cur]
+int mg_postsmooth(const erem_ctx* c, int l, const PcPoly& poly, int cur, const Geo& cg, const float* x_c,
+                  float omega, cudaStream_t s) {
+  const MgL L = mg_level(c, l);
+  const MgLevel& m = c->mg[l];
+  const int nb = grid_for(c, L.g.N);
+  int nxt = (cur + 1) % 3, prev = (cur + 2) % 3;
+  ++c->launches;
+  k_mg_prolong_sweep<<<nb, NT, 0, s>>>(L, m.rhs, m.x[cur], cg, x_c, omega,
+                                       poly.deg > 1 ? m.x[prev] : nullptr, m.x[nxt], (float)poly.c1[0],
+                                       (float)poly.c2[0]);
+  cur = nxt;
+  for (int j = 1; j < poly.deg; ++j) {
+    nxt = 3 - cur - prev;   // the third buffer
+    ++c->launches;
+    k_mg_sweep<<<nb, NT, 0, s>>>(L, m.rhs, m.x[prev], m.x[cur], m.x[nxt], (float)poly.c1[j],
+                                 (float)poly.c2[j]);
+    prev = cur;
+    cur = nxt;
+  }
+  return cur;
+}
+
+// Shared memory (floats) of levels l .. of the pressure multigrid in k_mg_small
+// (0: they do not fit), with the offsets of their arrays.
+int mg_small_plan(const erem_ctx* c, int l, MgSmall* A) {
+  const MgLevel& last = c->mg.back();
+  const int NC = last.nx * last.ny * last.nz;
+  A->n = (int)c->mg.size() - l;
+  if (!last.inv || NC > kMgCoarseThreads || A->n < 2 || A->n > kSmallLevels) return 0;
+  long long off = 0;
+  for (int k = 0; k < A->n; ++k) {
+    A->L[k] = mg_level(c, l + k);
+    A->off[k] = (int)off;
+    off += (long long)A->L[k].g.N * (c->dim == 3 ? 8 : 7) + coord_floats(A->L[k].g.N);
+    if (bits_of(A->L[k].g.nx) + bits_of(A->L[k].g.ny) + bits_of(A->L[k].g.nz) > 16) return 0;
+    if (off * 4 > c->smem_optin) return 0;
+  }
+  const int per = (NC + kSmallCtas - 1) / kSmallCtas;
+  A->inv_off = (int)off;
+  A->inv_stride = per | 1;   // odd: consecutive columns in other banks
+  off += (long long)NC * A->inv_stride + NC;
+  return off * 4 + 1024 <= c->smem_optin ? (int)off : 0;
+}
+
+template <typename Arg>
+void launch_small(const erem_ctx* c, void (*kern)(Arg), const Arg& A, int ctas, int floats, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(kSmallThreads);
+  cfg.dynamicSmemBytes = (size_t)floats * 4;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = ctas;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  ++c->launches;
+  cudaLaunchKernelEx(&cfg, kern, A);
 }
 
 // V-cycle below the fine level: the correction of coarse level l for its rhs
@@ -3340,6 +3910,23 @@ int mg_smooth(const erem_ctx* c, int l, const PcPoly& poly, int cur, bool from_z
 int mg_cycle(const erem_ctx* c, int l, const PcPoly& poly, float omega, cudaStream_t s) {
   const MgLevel& m = c->mg[l];
   const MgL L = mg_level(c, l);
+  if (c->mg_small && poly.deg <= 16) {
+    MgSmall A{};
+    if (const int floats = mg_small_plan(c, l, &A)) {
+      A.rhs = m.rhs;
+      A.x = m.x[0];
+      A.inv = c->mg.back().inv;
+      A.nu = poly.deg;
+      for (int j = 0; j < poly.deg; ++j) {
+        A.c1[j] = (float)poly.c1[j];
+        A.c2[j] = (float)poly.c2[j];
+      }
+      A.omega = omega;
+      A.ctrl = c->ctrl;
+      launch_small(c, k_mg_small, A, kSmallCtas, floats, s);
+      return 0;
+    }
+  }
   if (l + 1 == (int)c->mg.size()) {
     ++c->launches;
     if (m.inv && L.g.N <= kMgCoarseThreads && L.g.Np == L.g.N)
@@ -3352,14 +3939,12 @@ int mg_cycle(const erem_ctx* c, int l, const PcPoly& poly, float omega, cudaStre
                                                      kMgCoarseRtol);
     return 0;
   }
-  int cur = mg_smooth(c, l, poly, 0, true, s);
+  const int cur = mg_presmooth(c, l, poly, s);
   const MgL Lc = mg_level(c, l + 1);
   ++c->launches;
   k_mg_restrict<<<grid_for(c, Lc.g.N), NT, 0, s>>>(L, m.rhs, m.x[cur], Lc, c->mg[l + 1].rhs);
   const int ec = mg_cycle(c, l + 1, poly, omega, s);
-  ++c->launches;
-  k_mg_prolong<<<grid_for(c, L.g.N), NT, 0, s>>>(L, m.x[cur], Lc, c->mg[l + 1].x[ec], omega);
-  return mg_smooth(c, l, poly, cur, false, s);
+  return mg_postsmooth(c, l, poly, cur, Lc.g, c->mg[l + 1].x[ec], omega, s);
 }
 }  // namespace
 
@@ -3492,6 +4077,30 @@ constexpr int kSmgCoarseSweeps = 40;
 int smg_cycle(const erem_ctx* c, int l, cudaStream_t s) {
   const SmgLevel& m = c->smg[l];
   const MgN L = smg_level(c, l);
+  const SmgLevel& last = c->smg.back();
+  if (l > 0 && c->mg_small && (int)c->smg.size() - l >= 2 && (int)c->smg.size() - l <= kSmallLevels &&
+      last.nx * last.ny * last.nz <= 512) {
+    SmgSmall A{};
+    A.n = (int)c->smg.size() - l;
+    long long off = 0;
+    for (int k = 0; k < A.n; ++k) {
+      A.L[k] = smg_level(c, l + k);
+      A.off[k] = (int)off;
+      const Geo& g = A.L[k].g;
+      off += (long long)g.N * (c->dim == 3 ? 11 : 9) + coord_floats(g.N);
+      if (bits_of(g.nx) + bits_of(g.ny) + bits_of(g.nz) > 16) off = c->smem_optin;
+      if (off * 4 + 6144 > c->smem_optin) break;
+    }
+    if (off * 4 + 6144 <= c->smem_optin) {
+      A.rhs = m.rhs;
+      A.x = m.x[0];
+      A.sweeps = kSmgCoarseSweeps;
+      A.w = kSmgW;
+      A.ctrl = c->ctrl;
+      launch_small(c, k_smg_small, A, 1, (int)off, s);
+      return 0;
+    }
+  }
   if (l + 1 == (int)c->smg.size()) {
     ++c->launches;
     if (L.g.Np <= 512)
@@ -3501,16 +4110,14 @@ int smg_cycle(const erem_ctx* c, int l, cudaStream_t s) {
     return 0;
   }
   const int nb = grid_for(c, L.g.N);
-  c->launches += 2;
-  k_smg_jacobi<<<nb, NT, 0, s>>>(L, m.rhs, nullptr, m.x[0], kSmgW);
-  k_smg_jacobi<<<nb, NT, 0, s>>>(L, m.rhs, m.x[0], m.x[1], kSmgW);
+  ++c->launches;
+  k_smg_jacobi2<<<nb, NT, 0, s>>>(L, m.rhs, m.x[1], kSmgW);
   const MgN Lc = smg_level(c, l + 1);
   ++c->launches;
   k_smg_restrict<<<grid_for(c, Lc.g.N), NT, 0, s>>>(L, m.rhs, m.x[1], Lc, c->smg[l + 1].rhs);
   const int ec = smg_cycle(c, l + 1, s);
-  c->launches += 3;
-  k_smg_prolong<<<nb, NT, 0, s>>>(L.g, m.x[1], Lc.g, c->smg[l + 1].x[ec]);
-  k_smg_jacobi<<<nb, NT, 0, s>>>(L, m.rhs, m.x[1], m.x[2], kSmgW);
+  c->launches += 2;
+  k_smg_prolong_jacobi<<<nb, NT, 0, s>>>(L, m.rhs, m.x[1], Lc.g, c->smg[l + 1].x[ec], m.x[2], kSmgW);
   k_smg_jacobi<<<nb, NT, 0, s>>>(L, m.rhs, m.x[2], m.x[0], kSmgW);
   return 0;
 }
