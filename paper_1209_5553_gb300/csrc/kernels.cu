@@ -2749,6 +2749,7 @@ __global__ void k_bicg_init(JIn J, BiArr a, const double* __restrict__ b, double
       ctrl->lin[K_RHO_PREV] = 1.0;
       ctrl->lin[K_ALPHA] = 1.0;
       ctrl->lin[K_OMEGA] = 1.0;
+      ctrl->lin[K_BETA] = s;   // (rho / rho_prev) (alpha / omega)
       ctrl->lin[K_RR] = s;
       ctrl->lin[K_TOL2] = tol * tol * s;
       ctrl->lin_it = 0;
@@ -2761,9 +2762,7 @@ __global__ void k_bicg_init(JIn J, BiArr a, const double* __restrict__ b, double
 // p = r + beta (p - omega v); y = p / diag(A)
 __global__ void k_bicg_p(BiArr a, Geo g, Ctrl* ctrl) {
   if (*(volatile int*)&ctrl->lin_done) return;
-  const double* L = ctrl->lin;
-  const double beta = (L[K_RHO] / L[K_RHO_PREV]) * (L[K_ALPHA] / L[K_OMEGA]);
-  const double omega = L[K_OMEGA];
+  const double beta = ctrl->lin[K_BETA], omega = ctrl->lin[K_OMEGA];
   for (int i = blockIdx.x * NT + threadIdx.x; i < g.N; i += gridDim.x * NT) {
     int ix, iy, iz, ip;
     cell_of(i, g, ix, iy, iz, ip);
@@ -2884,6 +2883,9 @@ __global__ void k_bicg_r(BiArr a, Geo g, double* part, unsigned* cnt, Ctrl* ctrl
     if (threadIdx.x == 0) {
       *cnt = 0;
       ctrl->lin_it += 1;
+      // the next direction's beta, once: formed by every thread, its two FP64
+      // divisions were most of the direction pass
+      ctrl->lin[K_BETA] = (s0 / ctrl->lin[K_RHO]) * (ctrl->lin[K_ALPHA] / ctrl->lin[K_OMEGA]);
       ctrl->lin[K_RHO_PREV] = ctrl->lin[K_RHO];
       ctrl->lin[K_RHO] = s0;
       ctrl->lin[K_RR] = s1;
@@ -3268,9 +3270,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_smg_small(const __grid_con
 // FP64 (y, z of the Jacobi form)
 __global__ void k_bicg_p_mg(BiArr a, float* __restrict__ p32, Geo g, Ctrl* ctrl) {
   if (*(volatile int*)&ctrl->lin_done) return;
-  const double* L = ctrl->lin;
-  const double beta = (L[K_RHO] / L[K_RHO_PREV]) * (L[K_ALPHA] / L[K_OMEGA]);
-  const double omega = L[K_OMEGA];
+  const double beta = ctrl->lin[K_BETA], omega = ctrl->lin[K_OMEGA];
   for (int i = blockIdx.x * NT + threadIdx.x; i < g.N; i += gridDim.x * NT) {
     int ix, iy, iz, ip;
     cell_of(i, g, ix, iy, iz, ip);
@@ -3372,6 +3372,13 @@ BiArr bi_arr(const erem_ctx* c) {
 }
 
 int blocks_cells(const erem_ctx* c) { return grid_for(c, c->N); }
+// BiCGSTAB passes: a block's sum takes five FP64 operations per thread, as much
+// as the cells' own where every thread has one, so a thread takes up to four
+// cells while there are two blocks per SM (512^2: the five passes of an
+// iteration 66 -> 42 us, 9 of them from forming beta once)
+int blocks_bicg(const erem_ctx* c) {
+  return std::min(grid_for(c, c->N), std::max(2 * c->sm_count, grid_for(c, c->N / 4)));
+}
 int blocks_padded(const erem_ctx* c) { return grid_for(c, c->Np); }
 
 }  // namespace
@@ -4135,7 +4142,7 @@ void launch_smg_setup(const erem_ctx* c, double sigma, cudaStream_t s) {
 }
 
 void launch_bicg_iter_mg(const erem_ctx* c, double sigma, cudaStream_t s) {
-  const int nb = blocks_cells(c);
+  const int nb = blocks_bicg(c);
   const Geo g = geo_of(c);
   BiArr a = bi_arr(c);
   float* rhs0 = c->smg[0].rhs;
@@ -4158,7 +4165,7 @@ void launch_bicg_iter_mg(const erem_ctx* c, double sigma, cudaStream_t s) {
 }
 
 void launch_bicg_iter(const erem_ctx* c, double sigma, cudaStream_t s) {
-  const int nb = blocks_cells(c);
+  const int nb = blocks_bicg(c);
   const Geo g = geo_of(c);
   BiArr a = bi_arr(c);
   ++c->launches;
