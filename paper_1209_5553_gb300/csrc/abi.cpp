@@ -1176,8 +1176,7 @@ erem_status run_krylov(erem_ctx* c, const double* src, const KrOpts& o, erem_kry
     int cur = 0;
     for (int j = 0; j < m; ++j) {
       launch_kr_matvec(c, w_in, c->kr_V[j], c->kr_w[cur], j, 0, s);
-      for (int i = 1; i <= j; ++i) launch_kr_orth(c, c->kr_w[cur], c->kr_V[i - 1], c->kr_V[i], i, j, 0, s);
-      launch_kr_orth(c, c->kr_w[cur], c->kr_V[j], c->kr_V[j], j + 1, j, 1, s);
+      launch_kr_orth(c, c->kr_w[cur], j, s);
       w_in = c->kr_w[cur];
       cur ^= 1;
     }

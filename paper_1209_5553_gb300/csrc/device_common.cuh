@@ -40,27 +40,32 @@ __device__ __forceinline__ double warp_max(double v) {
 // the FP64 pipe (two results a clock and SM) is what bounds these passes.  One
 // warp that reads the 256 terms from shared memory, four lanes to a warp's
 // terms, needs 12.  Which warp differs from block to block, since a warp's index
-// picks the quarter of the SM whose pipe it uses.  128^3 pressure: (z, r), (z, Ad)
-// sweep 26.1 -> 22.2 us, A d 40.6 -> 38.5; a Krylov orthogonalisation pass at
-// 112^3 15.2 -> 12.8.
-__device__ double block_sum256(double v, int tid) {
-  __shared__ double all[8 * 36], res;   // pitch 36: the four lanes of eight warps take different banks
-  const int warp = (int)((blockIdx.x * 0x9E3779B1u) >> 29);
+// picks the quarter of the SM whose pipe it uses.  128^3 pressure: A d
+// 40.6 -> 38.4 us, the last sweep with (z, r) and (z, Ad) 26.1 -> 22.2, and 19.9
+// with both sums together.
+// The NV sums of a pass go together: one wait for shared memory, each summed by a
+// warp of its own.  The results are valid in every thread.
+template <int NV>
+__device__ void block_sums256(double (&v)[NV], int tid) {
+  __shared__ double all[NV][8 * 36], res[NV];   // pitch 36: the four lanes of eight warps take different banks
+  const int warp = ((tid >> 5) + (int)((blockIdx.x * 0x9E3779B1u) >> 29)) & 7;
   __syncthreads();
-  all[(tid >> 5) * 36 + (tid & 31)] = v;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) all[k][(tid >> 5) * 36 + (tid & 31)] = v[k];
   __syncthreads();
-  if ((tid >> 5) == warp) {
-    const double* p = all + ((tid & 31) >> 2) * 36 + (tid & 3);
+  if (warp < NV) {
+    const double* p = all[warp] + ((tid & 31) >> 2) * 36 + (tid & 3);
     double a = ((p[0] + p[16]) + (p[8] + p[24])) + ((p[4] + p[20]) + (p[12] + p[28]));
     a += __shfl_xor_sync(0xffffffffu, a, 2);
     a += __shfl_xor_sync(0xffffffffu, a, 1);
     a += __shfl_xor_sync(0xffffffffu, a, 16);
     a += __shfl_xor_sync(0xffffffffu, a, 8);
     a += __shfl_xor_sync(0xffffffffu, a, 4);
-    if ((tid & 31) == 0) res = a;
+    if ((tid & 31) == 0) res[warp] = a;
   }
   __syncthreads();
-  return res;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) v[k] = res[k];
 }
 
 // Block-wide reduction over BS threads with linear index tid; the result is
@@ -68,7 +73,11 @@ __device__ double block_sum256(double v, int tid) {
 // (syncs before reusing smem).
 template <int OP, int BS>
 __device__ double block_reduce_t(double v, double* sh, int tid) {
-  if (OP == 0 && BS == 256) return block_sum256(v, tid);
+  if (OP == 0 && BS == 256) {
+    double s[1] = {v};
+    block_sums256<1>(s, tid);
+    return s[0];
+  }
   v = OP == 0 ? warp_sum(v) : (OP == 1 ? warp_min(v) : warp_max(v));
   __syncthreads();
   if ((tid & 31) == 0) sh[tid >> 5] = v;
@@ -113,6 +122,33 @@ __device__ double gather_partials_t(const double* part, int k, double* sh, int t
     v = OP == 0 ? v + x : (OP == 1 ? fmin(v, x) : fmax(v, x));
   }
   return block_reduce_t<OP, BS>(v, sh, tid);
+}
+
+// The sums of partials 0 .. NV - 1 over all blocks, in block order, in every
+// thread.  The only block that still runs waits here: a thread's loads go out
+// together, not one after the other's addition.
+template <int NV>
+__device__ void gather_sums(const double* part, double (&out)[NV]) {
+  constexpr int kBatch = 4;
+  const int tid = threadIdx.x, nblocks = gridDim.x;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) out[k] = 0.0;
+  for (int b0 = tid; b0 < nblocks; b0 += kBatch * NT) {
+    double x[kBatch][NV];
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q)
+      if (b0 + q * NT < nblocks) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) x[q][k] = __ldcg(part + (b0 + q * NT) * kRedSlots + k);
+      }
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q)
+      if (b0 + q * NT < nblocks) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) out[k] += x[q][k];
+      }
+  }
+  block_sums256<NV>(out, tid);
 }
 template <int OP>
 __device__ double gather_partials(const double* part, int k, double* sh) {

@@ -143,6 +143,8 @@ struct KrDev {
   double beta;      // ||r||_2 of the start vector
   double avnorm;    // ||J v_{m+1}||_2
   double btol;      // breakdown threshold on h_{j+1,j}
+  double hinv;      // 1 / h of the vector that the next matvec scales
+  double gram[kKrMax + 1];  // v_i . v_{i+1} for odd i
   int breakdown;    // first j with h_{j+1,j} <= btol, or -1
   int pad;
 };
@@ -463,8 +465,8 @@ void launch_unpack(const erem_ctx* c, const double* src, double* dst, cudaStream
 void launch_kr_norm0(const erem_ctx* c, const double* r, double btol, cudaStream_t s);
 void launch_kr_matvec(const erem_ctx* c, const double* w_in, double* v_out, double* w_out, int j,
                       int mode, cudaStream_t s);
-void launch_kr_orth(const erem_ctx* c, double* w, const double* vprev, const double* vi, int i,
-                    int j, int last, cudaStream_t s);
+// w orthogonal to v_0 .. v_j (the dot with v_0 came with the matvec), ||w||_2 -> h_{j+1,j}
+void launch_kr_orth(const erem_ctx* c, double* w, int j, cudaStream_t s);
 struct KrComb {
   const double* v[kKrMax + 1];
   double coef[kKrMax + 1];

@@ -11,6 +11,7 @@
 // the last block to finish (atomic ticket) sums the partials in block order
 // and writes the result into the control block.  Min/max reductions are
 // exact in any order.
+#include <type_traits>
 #include <cstdlib>
 #include <algorithm>
 #include <cstdint>
@@ -952,7 +953,9 @@ __device__ __forceinline__ void leja_term_body(const Tq* __restrict__ qi, Tq* __
   const double bs = block_reduce<0>(acc, sh);
   double vals[1] = {bs};
   if (publish_partials(part, cnt, vals, 1)) {
-    const double S = gather_partials<0>(part, 0, sh);
+    double sum[1];
+    gather_sums<1>(part, sum);
+    const double S = sum[0];
     if (threadIdx.x == 0) {
       *cnt = 0;
       stop_test(ctrl, m, dm, S);
@@ -1159,41 +1162,87 @@ __global__ void k_kr_norm0(const double* __restrict__ r, Geo g, double btol, dou
   }
   double vals[1] = {block_reduce<0>(acc, sh)};
   if (publish_partials(part, cnt, vals, 1)) {
-    const double s = gather_partials<0>(part, 0, sh);
+    double sum[1];
+    gather_sums<1>(part, sum);
+    const double s = sum[0];
     if (threadIdx.x == 0) {
       *cnt = 0;
       K->beta = sqrt(s);
+      K->hinv = K->beta > 0.0 ? div_newton(1.0, K->beta) : 0.0;
       K->btol = btol;
       K->breakdown = K->beta <= 0.0 ? 0 : -1;
     }
   }
 }
 
-// v_j = w_in / h (h = beta for j = 0, else h_{j,j-1}); w_out = J v_j.
-// mode 0: the partial dot w_out . v_0 -> H(0, j); mode 1: ||w_out||_2 -> avnorm.
-__global__ void k_kr_matvec(JIn J, const double* __restrict__ w_in, double* __restrict__ v_out,
-                            double* __restrict__ w_out, const double* __restrict__ v0, Geo g, int j,
-                            int mode, double* part, unsigned* cnt, KrDev* K, int rev) {
+constexpr int kKrBlocks = 4;   // per SM: the registers of two cells' operands in flight
+
+// v_j = w_in / h (h = beta for j = 0, else h_{j,j-1}, its inverse formed by the
+// pass that has h: a division per thread was a fifth of this pass's FP64
+// operations); w_out = J v_j.  FP64-bound (11 operations per cell, 28 us at 112^3):
+// 39.8 -> 35.2 us there with the next cell's operands loaded ahead.  mode 0: the partial dot w_out . v_0 -> H(0, j); mode 1: ||w_out||_2 -> avnorm.
+__global__ void __launch_bounds__(NT, kKrBlocks)
+    k_kr_matvec(JIn J, const double* __restrict__ w_in, double* __restrict__ v_out,
+                double* __restrict__ w_out, const double* __restrict__ v0, Geo g, int j, int mode,
+                double* part, unsigned* cnt, KrDev* K, int rev) {
   __shared__ double sh[NT / 32];
   if (*(volatile int*)&K->breakdown >= 0) return;
-  const double h = j == 0 ? K->beta : K->H[j * kKrMax + (j - 1)];
-  const double s = 1.0 / h;
+  const double s = K->hinv;
   double acc = 0.0;
-  for (int idx = blockIdx.x * NT + threadIdx.x; idx < g.Np; idx += gridDim.x * NT) {
+  const bool dot0 = mode == 0 && j > 0;
+  struct In { double c[7], x[7], d; };
+  // the couplings out of the grid and of pad cells are 0 and their neighbours
+  // are not read
+  auto load = [&](int idx) {
     const int ip = kr_index(idx, g.Np, rev);
     int ix, iy, iz;
     kr_cell(ip, g, ix, iy, iz);
-    const double vc = s * w_in[ip];
+    In r;
+    r.c[0] = J.c[0][ip];
+    r.x[0] = w_in[ip];
+    r.d = dot0 ? v0[ip] : 0.0;
+    auto nb = [&](int k, bool in, int at) {
+      r.c[k] = in ? J.c[k][ip] : 0.0;
+      r.x[k] = in ? w_in[at] : 0.0;
+    };
+    nb(1, ix > 0, ip - 1);
+    nb(2, ix < g.nx - 1, ip + 1);
+    nb(3, iy > 0, ip - g.px);
+    nb(4, iy < g.ny - 1, ip + g.px);
+    if (g.dim == 3) {
+      nb(5, iz > 0, ip - g.plane);
+      nb(6, iz < g.nz - 1, ip + g.plane);
+    }
+    return r;
+  };
+  const int step = gridDim.x * NT;
+  int idx = blockIdx.x * NT + threadIdx.x;
+  In next;
+  if (idx < g.Np) next = load(idx);
+  for (; idx < g.Np; idx += step) {
+    const In now = next;
+    if (idx + step < g.Np) next = load(idx + step);
+    const int ip = kr_index(idx, g.Np, rev);
+    const double vc = s * now.x[0];
     v_out[ip] = vc;
     // J v_j = s (J w_in): one scaling of the sum instead of one per operand
     // (ten FP64 operations per cell instead of fifteen)
-    const double a = s * japply_cell(J, w_in, ip, ix, iy, iz, g);
+    double a = now.c[0] * now.x[0];
+#pragma unroll
+    for (int k = 1; k < 5; ++k) a = fma(now.c[k], now.x[k], a);
+    if (g.dim == 3) {
+      a = fma(now.c[5], now.x[5], a);
+      a = fma(now.c[6], now.x[6], a);
+    }
+    a *= s;
     w_out[ip] = a;
-    acc = fma(a, mode == 0 ? (j == 0 ? vc : v0[ip]) : a, acc);
+    acc = fma(a, mode == 0 ? (j == 0 ? vc : now.d) : a, acc);
   }
   double vals[1] = {block_reduce<0>(acc, sh)};
   if (publish_partials(part, cnt, vals, 1)) {
-    const double d = gather_partials<0>(part, 0, sh);
+    double sum[1];
+    gather_sums<1>(part, sum);
+    const double d = sum[0];
     if (threadIdx.x == 0) {
       *cnt = 0;
       if (mode == 0) K->H[j] = d;   // H(0, j)
@@ -1202,32 +1251,92 @@ __global__ void k_kr_matvec(JIn J, const double* __restrict__ w_in, double* __re
   }
 }
 
-// w -= h_{i-1,j} v_{i-1}; then the partial dot w . v_i -> H(i, j), or for
-// the last pass ||w||_2 -> h_{j+1,j} (and the breakdown test).
-__global__ void k_kr_orth(double* __restrict__ w, const double* __restrict__ vprev,
-                          const double* __restrict__ vi, Geo g, int i, int j, int last,
+// w -= sum of h_{k,j} v_k over the NP vectors from v_p on; then the dots with
+// the NN vectors from v_i on -> H(i, j), H(i + 1, j), or for NN = 0 (the last
+// pass) ||w||_2 -> h_{j+1,j} (and the breakdown test).
+//
+// Two vectors to a pass: modified Gram-Schmidt takes the second dot after the
+// first vector is subtracted, (w - h_i v_i) . v_{i+1} = w . v_{i+1} - h_i (v_i .
+// v_{i+1}) (the low-synchronisation form of Swirydowicz, Langou, Ananthan, Yang
+// and Thomas, 2020), with v_i . v_{i+1} formed once per basis by the pass that
+// first uses the pair (gram).  A pair reads and writes six vectors instead of
+// eight.  A thread loads its next cells before it computes: with all the blocks
+// resident and few cells to a thread, they would all wait for memory, then all
+// for the FP64 pipe.  112^3 (11 MB a vector, 1.5 M cells): 18.7 to 20.4 us a
+// pair, 22.7 before its three sums went together; one vector to a pass took 12.8
+// a vector.  Measured against 6 vectors at the copy rate 10 us, 4 FP64
+// operations per cell 10 us: neither fully hides the other.
+template <int NP, int NN>
+__global__ void __launch_bounds__(NT, kKrBlocks) k_kr_orth(double* __restrict__ w, const double* __restrict__ vp0,
+                          const double* __restrict__ vp1, const double* __restrict__ vn0,
+                          const double* __restrict__ vn1, Geo g, int p, int i, int j, int gram,
                           double* part, unsigned* cnt, KrDev* K, int rev) {
-  __shared__ double sh[NT / 32];
   if (*(volatile int*)&K->breakdown >= 0) return;
-  const double h = K->H[(i - 1) * kKrMax + j];
-  double acc = 0.0;
-  for (int idx = blockIdx.x * NT + threadIdx.x; idx < g.Np; idx += gridDim.x * NT) {
-    const int ip = kr_index(idx, g.Np, rev);
-    const double x = w[ip] - h * vprev[ip];
-    w[ip] = x;
-    acc = fma(x, last ? x : vi[ip], acc);
+  const double h0 = K->H[p * kKrMax + j];
+  const double h1 = NP > 1 ? K->H[(p + 1) * kKrMax + j] : 0.0;
+  double d0 = 0.0, d1 = 0.0, gr = 0.0;
+  const int nv = g.Np / 2;
+  struct In { double2 x, a, b, n0, n1; };
+  auto load = [&](int idx) {
+    const int v = 2 * kr_index(idx, nv, rev);
+    auto ld = [&](const double* q) { return *reinterpret_cast<const double2*>(q + v); };
+    In r;
+    r.x = ld(w);
+    r.a = ld(vp0);
+    if (NP > 1) r.b = ld(vp1);
+    if (NN > 0) r.n0 = ld(vn0);
+    if (NN > 1) r.n1 = ld(vn1);
+    return r;
+  };
+  const int step = gridDim.x * NT;
+  int idx = blockIdx.x * NT + threadIdx.x;
+  In next;
+  if (idx < nv) next = load(idx);
+  for (; idx < nv; idx += step) {
+    const In now = next;
+    if (idx + step < nv) next = load(idx + step);
+    const int v = 2 * kr_index(idx, nv, rev);
+    double2 x = now.x;
+    const double2 a = now.a, b = now.b, n0 = now.n0, n1 = now.n1;
+    x.x = fma(-h0, a.x, x.x);
+    x.y = fma(-h0, a.y, x.y);
+    if (NP > 1) {
+      x.x = fma(-h1, b.x, x.x);
+      x.y = fma(-h1, b.y, x.y);
+    }
+    *reinterpret_cast<double2*>(w + v) = x;
+    d0 = fma(x.x, NN > 0 ? n0.x : x.x, d0);
+    d0 = fma(x.y, NN > 0 ? n0.y : x.y, d0);
+    if (NN > 1) {
+      d1 = fma(x.x, n1.x, d1);
+      d1 = fma(x.y, n1.y, d1);
+      if (gram) {
+        gr = fma(n0.x, n1.x, gr);
+        gr = fma(n0.y, n1.y, gr);
+      }
+    }
   }
-  double vals[1] = {block_reduce<0>(acc, sh)};
-  if (publish_partials(part, cnt, vals, 1)) {
-    const double d = gather_partials<0>(part, 0, sh);
+  constexpr int NS = NN > 1 ? 3 : 1;   // sums
+  double vals[NS];
+  vals[0] = d0;
+  if constexpr (NS > 1) { vals[1] = d1; vals[2] = gr; }
+  block_sums256<NS>(vals, threadIdx.x);
+  if (publish_partials(part, cnt, vals, NS)) {
+    gather_sums<NS>(part, vals);
+    const double s0 = vals[0], s1 = vals[NS - 2 > 0 ? 1 : 0], s2 = vals[NS - 1];
     if (threadIdx.x == 0) {
       *cnt = 0;
-      if (!last) {
-        K->H[i * kKrMax + j] = d;
+      if (NN > 0) {
+        K->H[i * kKrMax + j] = s0;
+        if (NN > 1) {
+          if (gram) K->gram[i] = s2;
+          K->H[(i + 1) * kKrMax + j] = fma(-s0, gram ? s2 : K->gram[i], s1);
+        }
       } else {
-        const double hn = sqrt(d);
+        const double hn = sqrt(s0);
         K->H[(j + 1) * kKrMax + j] = hn;
         if (hn <= K->btol) K->breakdown = j;
+        else K->hinv = div_newton(1.0, hn);
       }
     }
   }
@@ -1720,7 +1829,6 @@ __device__ __forceinline__ double pres_apply(const PresArr& a, const double* __r
 // preconditioners form their own, and skip the FP64 division)
 template <int JAC>
 __global__ void k_cg_init(PresArr a, Geo g, double tol, double* part, unsigned* cnt, Ctrl* ctrl) {
-  __shared__ double sh[NT / 32];
   double rz = 0.0, rr = 0.0, bb = 0.0;
   for (int i = blockIdx.x * NT + threadIdx.x; i < g.N; i += gridDim.x * NT) {
     int ix, iy, iz, ip;
@@ -1737,13 +1845,14 @@ __global__ void k_cg_init(PresArr a, Geo g, double tol, double* part, unsigned* 
     bb += a.b[ip] * a.b[ip];
   }
   double vals[3];
-  vals[0] = block_reduce<0>(rz, sh);
-  vals[1] = block_reduce<0>(rr, sh);
-  vals[2] = block_reduce<0>(bb, sh);
+  vals[0] = rz;
+  vals[1] = rr;
+  vals[2] = bb;
+  block_sums256<3>(vals, threadIdx.x);
   if (publish_partials(part, cnt, vals, 3)) {
-    const double a0 = gather_partials<0>(part, 0, sh);
-    const double a1 = gather_partials<0>(part, 1, sh);
-    const double a2 = gather_partials<0>(part, 2, sh);
+    double sum[3];
+    gather_sums<3>(part, sum);
+    const double a0 = sum[0], a1 = sum[1], a2 = sum[2];
     if (threadIdx.x == 0) {
       *cnt = 0;
       ctrl->lin[K_RZ] = a0;
@@ -1817,7 +1926,9 @@ __global__ void k_cg_dir(PresArr a, const double* __restrict__ d, Geo g, double*
   }
   double vals[1] = {block_reduce<0>(dad, sh)};
   if (publish_partials(part, cnt, vals, 1)) {
-    const double s = gather_partials<0>(part, 0, sh);
+    double sum[1];
+    gather_sums<1>(part, sum);
+    const double s = sum[0];
     if (threadIdx.x == 0) {
       *cnt = 0;
       ctrl->lin[K_DAD] = s;
@@ -1834,7 +1945,6 @@ __global__ void k_cg_dir(PresArr a, const double* __restrict__ d, Geo g, double*
 // x += alpha d, r -= alpha Ad, z = r / diag; rz_new, rr -> beta, convergence
 __global__ void k_cg_upd(PresArr a, const double* __restrict__ d, Geo g, double* part,
                          unsigned* cnt, Ctrl* ctrl) {
-  __shared__ double sh[NT / 32];
   if (*(volatile int*)&ctrl->lin_done) return;
   const double alpha = ctrl->lin[K_ALPHA];
   double rz = 0.0, rr = 0.0;
@@ -1849,11 +1959,12 @@ __global__ void k_cg_upd(PresArr a, const double* __restrict__ d, Geo g, double*
     rz += r * z;
     rr += r * r;
   }
-  double vals[2] = {block_reduce<0>(rz, sh), 0.0};
-  vals[1] = block_reduce<0>(rr, sh);
+  double vals[2] = {rz, rr};
+  block_sums256<2>(vals, threadIdx.x);
   if (publish_partials(part, cnt, vals, 2)) {
-    const double s0 = gather_partials<0>(part, 0, sh);
-    const double s1 = gather_partials<0>(part, 1, sh);
+    double sum[2];
+    gather_sums<2>(part, sum);
+    const double s0 = sum[0], s1 = sum[1];
     if (threadIdx.x == 0) {
       *cnt = 0;
       ctrl->lin_it += 1;
@@ -1904,7 +2015,6 @@ template <bool FIRST, bool LAST>
 __global__ void k_pc_sweep(PresArr a, PcArr p, const float* __restrict__ zprev,
                            const float* __restrict__ zcur, float* __restrict__ znew, float c1,
                            float c2, Geo g, double* part, unsigned* cnt, Ctrl* ctrl) {
-  __shared__ double sh[NT / 32];
   if (*(volatile int*)&ctrl->lin_done) return;
   double rz = 0.0, zad = 0.0;
   const int nvec = g.Np / 4;
@@ -1985,11 +2095,12 @@ __global__ void k_pc_sweep(PresArr a, PcArr p, const float* __restrict__ zprev,
     }
   }
   if (!LAST) return;
-  double vals[2] = {block_reduce<0>(rz, sh), 0.0};
-  vals[1] = block_reduce<0>(zad, sh);
+  double vals[2] = {rz, zad};
+  block_sums256<2>(vals, threadIdx.x);
   if (publish_partials(part, cnt, vals, 2)) {
-    const double s0 = gather_partials<0>(part, 0, sh);
-    const double s1 = gather_partials<0>(part, 1, sh);
+    double sum[2];
+    gather_sums<2>(part, sum);
+    const double s0 = sum[0], s1 = sum[1];
     if (threadIdx.x == 0) {
       *cnt = 0;
       const double beta = ctrl->lin_it == 0 ? 0.0 : -ctrl->lin[K_ALPHA] * s1 / ctrl->lin[K_RZ];
@@ -2627,7 +2738,9 @@ __global__ void k_pcg_upd(PresArr a, const double* __restrict__ d, Geo g, double
   }
   double vals[1] = {block_reduce<0>(rr, sh)};
   if (publish_partials(part, cnt, vals, 1)) {
-    const double s1 = gather_partials<0>(part, 0, sh);
+    double sum[1];
+    gather_sums<1>(part, sum);
+    const double s1 = sum[0];
     if (threadIdx.x == 0) {
       *cnt = 0;
       ctrl->lin_it += 1;
@@ -2650,7 +2763,9 @@ __global__ void k_sumsq(const double* __restrict__ x, Geo g, double* part, unsig
   }
   double vals[1] = {block_reduce<0>(s, sh)};
   if (publish_partials(part, cnt, vals, 1)) {
-    const double a = gather_partials<0>(part, 0, sh);
+    double sum[1];
+    gather_sums<1>(part, sum);
+    const double a = sum[0];
     if (threadIdx.x == 0) {
       *cnt = 0;
       ctrl->lin[K_EMB] = a;
@@ -2701,7 +2816,9 @@ __global__ void k_pres_post(const double* __restrict__ m, PresArr a, Geo g, Phys
   double vals[2] = {block_reduce<0>(fin, sh), 0.0};
   vals[1] = block_reduce<2>(vmax, sh);
   if (publish_partials(part, cnt, vals, 2)) {
-    const double s0 = gather_partials<0>(part, 0, sh);
+    double sum[1];
+    gather_sums<1>(part, sum);
+    const double s0 = sum[0];
     const double s1 = gather_partials<2>(part, 1, sh);
     if (threadIdx.x == 0) {
       *cnt = 0;
@@ -2741,7 +2858,9 @@ __global__ void k_bicg_init(JIn J, BiArr a, const double* __restrict__ b, double
   }
   double vals[1] = {block_reduce<0>(bb, sh)};
   if (publish_partials(part, cnt, vals, 1)) {
-    const double s = gather_partials<0>(part, 0, sh);
+    double sum[1];
+    gather_sums<1>(part, sum);
+    const double s = sum[0];
     if (threadIdx.x == 0) {
       *cnt = 0;
       ctrl->lin[K_BB] = s;
@@ -2787,7 +2906,9 @@ __global__ void k_bicg_v(JIn J, BiArr a, double sigma, Geo g, double* part, unsi
   }
   double vals[1] = {block_reduce<0>(rv, sh)};
   if (publish_partials(part, cnt, vals, 1)) {
-    const double s = gather_partials<0>(part, 0, sh);
+    double sum[1];
+    gather_sums<1>(part, sum);
+    const double s = sum[0];
     if (threadIdx.x == 0) {
       *cnt = 0;
       if (s == 0.0 || !isfinite(s)) {
@@ -2817,7 +2938,9 @@ __global__ void k_bicg_s(BiArr a, Geo g, double* part, unsigned* cnt, Ctrl* ctrl
   }
   double vals[1] = {block_reduce<0>(ss, sh)};
   if (publish_partials(part, cnt, vals, 1)) {
-    const double s = gather_partials<0>(part, 0, sh);
+    double sum[1];
+    gather_sums<1>(part, sum);
+    const double s = sum[0];
     if (threadIdx.x == 0) {
       *cnt = 0;
       ctrl->lin[K_SS] = s;
@@ -2833,7 +2956,6 @@ __global__ void k_bicg_s(BiArr a, Geo g, double* part, unsigned* cnt, Ctrl* ctrl
 // t = A z; omega = (t, s) / (t, t); x += omega z; r = s - omega t; new rho
 __global__ void k_bicg_t(JIn J, BiArr a, double sigma, Geo g, double* part, unsigned* cnt,
                          Ctrl* ctrl) {
-  __shared__ double sh[NT / 32];
   if (*(volatile int*)&ctrl->lin_done) return;
   double ts = 0.0, tt = 0.0;
   for (int i = blockIdx.x * NT + threadIdx.x; i < g.N; i += gridDim.x * NT) {
@@ -2844,11 +2966,12 @@ __global__ void k_bicg_t(JIn J, BiArr a, double sigma, Geo g, double* part, unsi
     ts += t * a.s[ip];
     tt += t * t;
   }
-  double vals[2] = {block_reduce<0>(ts, sh), 0.0};
-  vals[1] = block_reduce<0>(tt, sh);
+  double vals[2] = {ts, tt};
+  block_sums256<2>(vals, threadIdx.x);
   if (publish_partials(part, cnt, vals, 2)) {
-    const double s0 = gather_partials<0>(part, 0, sh);
-    const double s1 = gather_partials<0>(part, 1, sh);
+    double sum[2];
+    gather_sums<2>(part, sum);
+    const double s0 = sum[0], s1 = sum[1];
     if (threadIdx.x == 0) {
       *cnt = 0;
       if (s1 == 0.0 || !isfinite(s1) || s0 == 0.0) {
@@ -2862,7 +2985,6 @@ __global__ void k_bicg_t(JIn J, BiArr a, double sigma, Geo g, double* part, unsi
 }
 
 __global__ void k_bicg_r(BiArr a, Geo g, double* part, unsigned* cnt, Ctrl* ctrl) {
-  __shared__ double sh[NT / 32];
   if (*(volatile int*)&ctrl->lin_done) return;
   const double omega = ctrl->lin[K_OMEGA];
   double rho = 0.0, rr = 0.0;
@@ -2875,11 +2997,12 @@ __global__ void k_bicg_r(BiArr a, Geo g, double* part, unsigned* cnt, Ctrl* ctrl
     rho += a.rh[ip] * r;
     rr += r * r;
   }
-  double vals[2] = {block_reduce<0>(rho, sh), 0.0};
-  vals[1] = block_reduce<0>(rr, sh);
+  double vals[2] = {rho, rr};
+  block_sums256<2>(vals, threadIdx.x);
   if (publish_partials(part, cnt, vals, 2)) {
-    const double s0 = gather_partials<0>(part, 0, sh);
-    const double s1 = gather_partials<0>(part, 1, sh);
+    double sum[2];
+    gather_sums<2>(part, sum);
+    const double s0 = sum[0], s1 = sum[1];
     if (threadIdx.x == 0) {
       *cnt = 0;
       ctrl->lin_it += 1;
@@ -3297,7 +3420,9 @@ __global__ void k_bicg_s_mg(BiArr a, float* __restrict__ s32, Geo g, double* par
   }
   double vals[1] = {block_reduce<0>(ss, sh)};
   if (publish_partials(part, cnt, vals, 1)) {
-    const double s = gather_partials<0>(part, 0, sh);
+    double sum[1];
+    gather_sums<1>(part, sum);
+    const double s = sum[0];
     if (threadIdx.x == 0) {
       *cnt = 0;
       ctrl->lin[K_SS] = s;
@@ -3378,6 +3503,13 @@ int blocks_cells(const erem_ctx* c) { return grid_for(c, c->N); }
 // iteration 66 -> 42 us, 9 of them from forming beta once)
 int blocks_bicg(const erem_ctx* c) {
   return std::min(grid_for(c, c->N), std::max(2 * c->sm_count, grid_for(c, c->N / 4)));
+}
+// Blocks for `items`, one to a thread and pass of the grid's loop, with the same
+// number of passes in every thread
+int blocks_even(const erem_ctx* c, long long items, int per_sm) {
+  const long long full = (long long)NT * std::min(c->red_blocks, per_sm * c->sm_count);
+  const long long per = std::max(1LL, (items + full - 1) / full);
+  return grid_for(c, (items + per - 1) / per);
 }
 int blocks_padded(const erem_ctx* c) { return grid_for(c, c->Np); }
 
@@ -4206,15 +4338,41 @@ void launch_kr_norm0(const erem_ctx* c, const double* r, double btol, cudaStream
 void launch_kr_matvec(const erem_ctx* c, const double* w_in, double* v_out, double* w_out, int j,
                       int mode, cudaStream_t s) {
   ++c->launches;
-  k_kr_matvec<<<blocks_padded(c), NT, 0, s>>>(jin(c), w_in, v_out, w_out, c->kr_V[0], geo_of(c), j,
+  k_kr_matvec<<<blocks_even(c, c->Np, kKrBlocks), NT, 0, s>>>(jin(c), w_in, v_out, w_out, c->kr_V[0], geo_of(c), j,
                                               mode, c->red_part, c->red_cnt, c->kr_dev, kr_dir(c));
 }
 
-void launch_kr_orth(const erem_ctx* c, double* w, const double* vprev, const double* vi, int i,
-                    int j, int last, cudaStream_t s) {
-  ++c->launches;
-  k_kr_orth<<<blocks_padded(c), NT, 0, s>>>(w, vprev, vi, geo_of(c), i, j, last, c->red_part,
-                                            c->red_cnt, c->kr_dev, kr_dir(c));
+void launch_kr_orth(const erem_ctx* c, double* w, int j, cudaStream_t s) {
+  const int nb = blocks_even(c, c->Np / 2, kKrBlocks);
+  auto pass = [&](auto np, auto nn, int p, int i) {
+    constexpr int NP = decltype(np)::value, NN = decltype(nn)::value;
+    double* const* V = c->kr_V;
+    ++c->launches;
+    k_kr_orth<NP, NN><<<nb, NT, 0, s>>>(w, V[p], NP > 1 ? V[p + 1] : nullptr, NN > 0 ? V[i] : nullptr,
+                                        NN > 1 ? V[i + 1] : nullptr, geo_of(c), p, i, j, i + 1 == j,
+                                        c->red_part, c->red_cnt, c->kr_dev, kr_dir(c));
+  };
+  using One = std::integral_constant<int, 1>;
+  using Two = std::integral_constant<int, 2>;
+  using None = std::integral_constant<int, 0>;
+  // v_0's dot came with J v_j; then pairs from v_1 on, the pass of a pair
+  // subtracting the vectors of the one before
+  int p = 0, np = 1;
+  for (int i = 1; i <= j;) {
+    const int nn = i + 1 <= j ? 2 : 1;
+    if (np == 1) {
+      if (nn == 2) pass(One{}, Two{}, p, i);
+      else pass(One{}, One{}, p, i);
+    } else {
+      if (nn == 2) pass(Two{}, Two{}, p, i);
+      else pass(Two{}, One{}, p, i);
+    }
+    p = i;
+    np = nn;
+    i += nn;
+  }
+  if (np == 1) pass(One{}, None{}, p, j + 1);
+  else pass(Two{}, None{}, p, j + 1);
 }
 
 void launch_kr_combine(const erem_ctx* c, double* y, const KrComb& cb, cudaStream_t s) {
