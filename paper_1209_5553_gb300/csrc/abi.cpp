@@ -192,8 +192,6 @@ bool ensure_pcg_graph(erem_ctx* c, const PcPoly& P, const float* z) {
   const long long key = ((long long)c->pc_deg << 40) ^ ((long long)c->mg_nu << 32) ^
                         (long long)(c->mg_omega * 1e6f);
   if (c->pcg_exec && c->pcg_key == key) return true;
-  if (c->bicg_exec) cudaGraphExecDestroy(c->bicg_exec);
-  if (c->bicg_graph) cudaGraphDestroy(c->bicg_graph);
   if (c->pcg_exec) cudaGraphExecDestroy(c->pcg_exec);
   if (c->pcg_graph) cudaGraphDestroy(c->pcg_graph);
   c->pcg_exec = nullptr;
@@ -1453,6 +1451,8 @@ erem_status erem_destroy(erem_ctx* c) {
     if (p) cudaFree(p);
   for (float* p : c->pc)
     if (p) cudaFree(p);
+  if (c->bicg_exec) cudaGraphExecDestroy(c->bicg_exec);
+  if (c->bicg_graph) cudaGraphDestroy(c->bicg_graph);
   if (c->pcg_exec) cudaGraphExecDestroy(c->pcg_exec);
   if (c->pcg_graph) cudaGraphDestroy(c->pcg_graph);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
