@@ -2161,6 +2161,7 @@ __global__ void k_mg_coarsen(MgL f, MgL c) {
 }
 
 // (N x)_i: the couplings of cell i to its neighbours applied to x
+template <int DIM = 0>
 __device__ __forceinline__ float mg_offdiag(const MgL& L, const float* __restrict__ x, int ip, int ix,
                                             int iy, int iz) {
   float s = 0.0f;
@@ -2168,7 +2169,7 @@ __device__ __forceinline__ float mg_offdiag(const MgL& L, const float* __restric
   if (ix > 0) s = fmaf(L.Ux[ip - 1], x[ip - 1], s);
   if (iy < L.g.ny - 1) s = fmaf(L.Uy[ip], x[ip + L.g.px], s);
   if (iy > 0) s = fmaf(L.Uy[ip - L.g.px], x[ip - L.g.px], s);
-  if (L.g.dim == 3) {
+  if (DIM == 3 || (DIM == 0 && L.g.dim == 3)) {
     if (iz < L.g.nz - 1) s = fmaf(L.Uz[ip], x[ip + L.g.plane], s);
     if (iz > 0) s = fmaf(L.Uz[ip - L.g.plane], x[ip - L.g.plane], s);
   }
@@ -2247,21 +2248,36 @@ __global__ void k_mg_prolong_sweep(MgL L, const float* __restrict__ rhs, const f
   }
 }
 
-// rhs_c = P^T (rhs_f - A_f x_f)
+// rhs_c = P^T (rhs_f - A_f x_f).  In 2D the four
+// children are unrolled, so that their loads go out together (512^2 and below
+// 2.9 -> 2.5 us a level); the eight of 3D are not (128^3 7.0 us, unrolled 7.9).
+template <int DIM>
 __global__ void k_mg_restrict(MgL f, const float* __restrict__ rhs_f, const float* __restrict__ x_f,
                               MgL c, float* __restrict__ rhs_c) {
   for (int I = blockIdx.x * NT + threadIdx.x; I < c.g.N; I += gridDim.x * NT) {
     int X, Y, Z, IP;
     cell_of(I, c.g, X, Y, Z, IP);
-    const int xe = min(2 * X + 2, f.g.nx), ye = min(2 * Y + 2, f.g.ny);
-    const int ze = f.g.dim == 3 ? min(2 * Z + 2, f.g.nz) : 1;
     float acc = 0.0f;
-    for (int iz = (f.g.dim == 3 ? 2 * Z : 0); iz < ze; ++iz)
-      for (int iy = 2 * Y; iy < ye; ++iy)
-        for (int ix = 2 * X; ix < xe; ++ix) {
-          const int ip = ix + f.g.px * (iy + f.g.ny * iz);
-          acc += rhs_f[ip] - fmaf(f.diag[ip], x_f[ip], -mg_offdiag(f, x_f, ip, ix, iy, iz));
+    if constexpr (DIM == 2) {
+#pragma unroll
+      for (int ky = 0; ky < 2; ++ky)
+#pragma unroll
+        for (int kx = 0; kx < 2; ++kx) {
+          const int ix = 2 * X + kx, iy = 2 * Y + ky, iz = 0;
+          if (ix < f.g.nx && iy < f.g.ny) {
+            const int ip = ix + f.g.px * iy;
+            acc += rhs_f[ip] - fmaf(f.diag[ip], x_f[ip], -mg_offdiag<DIM>(f, x_f, ip, ix, iy, iz));
+          }
         }
+    } else {
+      const int xe = min(2 * X + 2, f.g.nx), ye = min(2 * Y + 2, f.g.ny), ze = min(2 * Z + 2, f.g.nz);
+      for (int iz = 2 * Z; iz < ze; ++iz)
+        for (int iy = 2 * Y; iy < ye; ++iy)
+          for (int ix = 2 * X; ix < xe; ++ix) {
+            const int ip = ix + f.g.px * (iy + f.g.ny * iz);
+            acc += rhs_f[ip] - fmaf(f.diag[ip], x_f[ip], -mg_offdiag<DIM>(f, x_f, ip, ix, iy, iz));
+          }
+    }
     rhs_c[IP] = acc;
   }
 }
@@ -2517,9 +2533,13 @@ __device__ __forceinline__ SmallCell fill_cells(const Geo& g, float* at, int tid
   c.by = bits_of(g.ny);
   unsigned short* co = reinterpret_cast<unsigned short*>(at);
   c.co = co;
+  // i / n as (i ceil(2^32 / n)) >> 32, exact for i, n up to 2^13: one 32-bit
+  // division per dimension and thread instead of three per cell
+  const unsigned mx = 0xffffffffu / (unsigned)g.nx + 1u, my = 0xffffffffu / (unsigned)g.ny + 1u;
   for (int i = tid; i < g.N; i += threads) {
-    int ix, iy, iz, ip;
-    cell_of(i, g, ix, iy, iz, ip);
+    const int row = g.nx > 1 ? (int)__umulhi((unsigned)i, mx) : i;
+    const int iz = g.ny > 1 ? (int)__umulhi((unsigned)row, my) : row;
+    const int ix = i - row * g.nx, iy = row - iz * g.ny;
     co[i] = (unsigned short)(ix | (iy << c.bx) | (iz << (c.bx + c.by)));
   }
   return c;
@@ -2591,7 +2611,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_mg_small(const __grid_cons
       float *rhs, *xa, *xb;
       const MgL S = level(l, rhs, xa, xb);
       const MgL& G = A.L[l];
-      if (l + 1 < A.n)
+      if (l + 1 < A.n) {
+#pragma unroll 4
         for (int i = tid; i < G.g.N; i += kSmallThreads) {
           S.dinv[i] = G.dinv[i];
           S.diag[i] = G.diag[i];
@@ -2599,13 +2620,17 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_mg_small(const __grid_cons
           S.Uy[i] = G.Uy[i];
           if (G.g.dim == 3) S.Uz[i] = G.Uz[i];
         }
+      }
       if (l == 0)
         for (int i = tid; i < G.g.N; i += kSmallThreads) rhs[i] = A.rhs[i];
       fill_cells(G.g, sm + A.off[l] + (G.g.dim == 3 ? 8 : 7) * G.g.N, tid, kSmallThreads);
     }
   }
-  for (int k = tid; k < NC * (i1 - i0); k += kSmallThreads) {
-    const int j = k / (i1 - i0), i = k - j * (i1 - i0);
+  const int own = i1 - i0;
+  const unsigned mo = own > 1 ? 0xffffffffu / (unsigned)own + 1u : 0u;   // as in fill_cells
+#pragma unroll 4
+  for (int k = tid; k < NC * own; k += kSmallThreads) {
+    const int j = own > 1 ? (int)__umulhi((unsigned)k, mo) : k, i = k - j * own;
     inv[j * A.inv_stride + i] = A.inv[(size_t)j * NC + i0 + i];
   }
   __syncthreads();
@@ -3038,6 +3063,7 @@ struct MgN {
   Geo g;
 };
 
+template <int DIM = 0>
 __device__ __forceinline__ float smg_offdiag(const MgN& L, const float* __restrict__ x, int ip, int ix,
                                              int iy, int iz) {
   float s = 0.0f;
@@ -3045,7 +3071,7 @@ __device__ __forceinline__ float smg_offdiag(const MgN& L, const float* __restri
   if (ix < L.g.nx - 1) s = fmaf(L.c[1][ip], x[ip + 1], s);
   if (iy > 0) s = fmaf(L.c[2][ip], x[ip - L.g.px], s);
   if (iy < L.g.ny - 1) s = fmaf(L.c[3][ip], x[ip + L.g.px], s);
-  if (L.g.dim == 3) {
+  if (DIM == 3 || (DIM == 0 && L.g.dim == 3)) {
     if (iz > 0) s = fmaf(L.c[4][ip], x[ip - L.g.plane], s);
     if (iz < L.g.nz - 1) s = fmaf(L.c[5][ip], x[ip + L.g.plane], s);
   }
@@ -3154,21 +3180,36 @@ __global__ void k_smg_prolong_jacobi(MgN L, const float* __restrict__ rhs, const
   }
 }
 
-// rhs_c = P^T (rhs_f - A_f x_f)
+// rhs_c = P^T (rhs_f - A_f x_f).  In 2D the four
+// children are unrolled, so that their loads go out together (512^2 and below
+// 2.9 -> 2.5 us a level); the eight of 3D are not (128^3 7.0 us, unrolled 7.9).
+template <int DIM>
 __global__ void k_smg_restrict(MgN f, const float* __restrict__ rhs_f, const float* __restrict__ x_f,
-                               MgN c, float* __restrict__ rhs_c) {
+                              MgN c, float* __restrict__ rhs_c) {
   for (int I = blockIdx.x * NT + threadIdx.x; I < c.g.N; I += gridDim.x * NT) {
     int X, Y, Z, IP;
     cell_of(I, c.g, X, Y, Z, IP);
-    const int xe = min(2 * X + 2, f.g.nx), ye = min(2 * Y + 2, f.g.ny);
-    const int ze = f.g.dim == 3 ? min(2 * Z + 2, f.g.nz) : 1;
     float acc = 0.0f;
-    for (int iz = (f.g.dim == 3 ? 2 * Z : 0); iz < ze; ++iz)
-      for (int iy = 2 * Y; iy < ye; ++iy)
-        for (int ix = 2 * X; ix < xe; ++ix) {
-          const int ip = ix + f.g.px * (iy + f.g.ny * iz);
-          acc += rhs_f[ip] - fmaf(f.D[ip], x_f[ip], -smg_offdiag(f, x_f, ip, ix, iy, iz));
+    if constexpr (DIM == 2) {
+#pragma unroll
+      for (int ky = 0; ky < 2; ++ky)
+#pragma unroll
+        for (int kx = 0; kx < 2; ++kx) {
+          const int ix = 2 * X + kx, iy = 2 * Y + ky, iz = 0;
+          if (ix < f.g.nx && iy < f.g.ny) {
+            const int ip = ix + f.g.px * iy;
+            acc += rhs_f[ip] - fmaf(f.D[ip], x_f[ip], -smg_offdiag<DIM>(f, x_f, ip, ix, iy, iz));
+          }
         }
+    } else {
+      const int xe = min(2 * X + 2, f.g.nx), ye = min(2 * Y + 2, f.g.ny), ze = min(2 * Z + 2, f.g.nz);
+      for (int iz = 2 * Z; iz < ze; ++iz)
+        for (int iy = 2 * Y; iy < ye; ++iy)
+          for (int ix = 2 * X; ix < xe; ++ix) {
+            const int ip = ix + f.g.px * (iy + f.g.ny * iz);
+            acc += rhs_f[ip] - fmaf(f.D[ip], x_f[ip], -smg_offdiag<DIM>(f, x_f, ip, ix, iy, iz));
+          }
+    }
     rhs_c[IP] = acc;
   }
 }
@@ -3304,6 +3345,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_smg_small(const __grid_con
     const MgN S = level(l, rhs, xa, xb);
     const MgN& G = A.L[l];
     const int nk = G.g.dim == 3 ? 6 : 4;
+#pragma unroll 4
     for (int i = tid; i < G.g.N; i += kSmallThreads) {
       S.D[i] = G.D[i];
       S.Dinv[i] = G.Dinv[i];
@@ -4081,7 +4123,7 @@ int mg_cycle(const erem_ctx* c, int l, const PcPoly& poly, float omega, cudaStre
   const int cur = mg_presmooth(c, l, poly, s);
   const MgL Lc = mg_level(c, l + 1);
   ++c->launches;
-  k_mg_restrict<<<grid_for(c, Lc.g.N), NT, 0, s>>>(L, m.rhs, m.x[cur], Lc, c->mg[l + 1].rhs);
+  (c->dim == 3 ? k_mg_restrict<3> : k_mg_restrict<2>)<<<grid_for(c, Lc.g.N), NT, 0, s>>>(L, m.rhs, m.x[cur], Lc, c->mg[l + 1].rhs);
   const int ec = mg_cycle(c, l + 1, poly, omega, s);
   return mg_postsmooth(c, l, poly, cur, Lc.g, c->mg[l + 1].x[ec], omega, s);
 }
@@ -4117,7 +4159,7 @@ const float* launch_pc_apply(const erem_ctx* c, const PcPoly& poly, cudaStream_t
     const MgL F = mg_fine(c);
     const MgL C1 = mg_level(c, 0);
     ++c->launches;
-    k_mg_restrict<<<grid_for(c, C1.g.N), NT, 0, s>>>(F, p.r, zb[x0], C1, c->mg[0].rhs);
+    (c->dim == 3 ? k_mg_restrict<3> : k_mg_restrict<2>)<<<grid_for(c, C1.g.N), NT, 0, s>>>(F, p.r, zb[x0], C1, c->mg[0].rhs);
     const int ec = mg_cycle(c, 0, poly, c->mg_omega, s);
     ++c->launches;
     k_mg_prolong<<<blocks_cells(c), NT, 0, s>>>(F, zb[x0], C1, c->mg[0].x[ec], c->mg_omega);
@@ -4253,7 +4295,7 @@ int smg_cycle(const erem_ctx* c, int l, cudaStream_t s) {
   k_smg_jacobi2<<<nb, NT, 0, s>>>(L, m.rhs, m.x[1], kSmgW);
   const MgN Lc = smg_level(c, l + 1);
   ++c->launches;
-  k_smg_restrict<<<grid_for(c, Lc.g.N), NT, 0, s>>>(L, m.rhs, m.x[1], Lc, c->smg[l + 1].rhs);
+  (c->dim == 3 ? k_smg_restrict<3> : k_smg_restrict<2>)<<<grid_for(c, Lc.g.N), NT, 0, s>>>(L, m.rhs, m.x[1], Lc, c->smg[l + 1].rhs);
   const int ec = smg_cycle(c, l + 1, s);
   c->launches += 2;
   k_smg_prolong_jacobi<<<nb, NT, 0, s>>>(L, m.rhs, m.x[1], Lc.g, c->smg[l + 1].x[ec], m.x[2], kSmgW);
