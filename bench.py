@@ -66,6 +66,52 @@ def term_bytes_per_cell(full_bytes: int, degrees, lagged: bool = False) -> float
         odd = m if lagged else (m + 1) // 2
         total += odd * full_bytes + (m - odd) * (full_bytes - P_BYTES)
     return float(total)
+
+
+def term_form(n_launches: int, n_terms: int) -> str:
+    """How the timed Leja terms ran, from the launches they took: "resident"
+    (all terms of a substep in one launch, the working set on the chip), "pair"
+    (two terms to a launch) or "single"."""
+    if not n_terms or n_launches >= 0.95 * n_terms:
+        return "single"
+    return "pair" if n_launches >= 0.45 * n_terms else "resident"
+
+
+def leja_bytes(form: str, full_bytes: int, degrees, lagged: bool):
+    """Algorithmic HBM bytes per cell of all Leja terms in this form: a pair
+    reads the coefficients, q and P once and writes q and P once (the odd-term
+    bytes) for two terms; the resident form keeps all of them on the chip, so
+    it has none to speak of (None)."""
+    if form == "resident":
+        return None
+    if form == "pair":
+        return float(sum((m + 1) // 2 * full_bytes for m in degrees))
+    return term_bytes_per_cell(full_bytes, degrees, lagged)
+
+
+def leja_roofline(form: str, fp: str, dim: int, full_bytes: int, degrees, lagged, cells, t_ms, n_terms,
+                  n_launches, peak, peak_source):
+    """The roofline object of the Leja kernel that ran."""
+    vec = 4 if fp == "float" else 2
+    bpc = leja_bytes(form, full_bytes, degrees, lagged)
+    ach = bpc * cells / (t_ms / 1e3) / 1e9 if bpc and t_ms else None
+    r = {"kernel": {"single": f"k_leja_term<{fp},{vec},{dim}>", "pair": "k_leja_pair",
+                    "resident": f"k_leja_res<{fp},{vec},{dim}>"}[form],
+         "form": form, "bound": {"single": "hbm", "pair": "latency and hbm", "resident": "latency"}[form],
+         "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak if ach else None, "traffic": None,
+         "peak_source": peak_source, "terms_lagged": lagged,
+         "terms_per_launch": n_terms / max(n_launches, 1), "term_ms_avg": t_ms / max(n_terms, 1)}
+    if form == "single":
+        r["algorithmic_bytes_per_cell"] = {"odd_terms": full_bytes,
+                                           "even_terms": full_bytes if lagged else full_bytes - P_BYTES}
+    elif form == "pair":
+        r["algorithmic_bytes_per_cell"] = {"pair_of_terms": full_bytes}
+    else:
+        r["note"] = ("coefficients, Newton vectors and P stay in shared memory and registers for all terms "
+                     "of a substep: no HBM rate")
+    return r
+
+
 FALLBACK_HBM_GBS = 6800.0
 
 
@@ -205,25 +251,29 @@ def measured_peaks():
         return FALLBACK_HBM_GBS, "fallback"
 
 
-def kernel_sources_sha():
-    """Hash of the source the Leja term kernel is built from: the shared
-    device helpers and the k_leja_term body and entry points."""
+def kernel_sources_sha(form: str):
+    """Hash of the source the Leja kernel of this form is built from: the shared
+    device helpers and the k_leja_term body and entry points, or the pair's file."""
     csrc = os.path.join(ROOT, "paper_1209_5553_gb300", "csrc")
-    kern = open(os.path.join(csrc, "kernels.cu")).read()
-    start = kern.index("__device__ __forceinline__ void leja_term_body(")
-    end = kern.index("\n}\n", kern.index("k_leja_term1(const Tq* __restrict__ qi", start))
     h = hashlib.sha256()
     h.update(open(os.path.join(csrc, "device_common.cuh"), "rb").read())
-    h.update(kern[start:end].encode())
+    if form == "pair":
+        h.update(open(os.path.join(csrc, "leja_pair.cu"), "rb").read())
+    else:
+        kern = open(os.path.join(csrc, "kernels.cu")).read()
+        start = kern.index("__device__ __forceinline__ void leja_term_body(")
+        end = kern.index("\n}\n", kern.index("k_leja_term1(const Tq* __restrict__ qi", start))
+        h.update(kern[start:end].encode())
     return h.hexdigest()[:16]
 
 
-def recorded_traffic(precision: str, n_cells: int):
-    """Bytes per Leja-term launch from the committed ncu summary, if it was
-    taken on the current kernel source (else None)."""
-    path = os.path.join(ROOT, "profiles", f"k_leja_term_{precision}_channels3d_{round(n_cells ** (1 / 3))}.md")
+def recorded_traffic(form: str, precision: str, n_cells: int):
+    """Bytes per Leja launch (a term, or a pair of terms) from the committed ncu
+    summary, if it was taken on the current kernel source (else None)."""
+    name = {"single": "k_leja_term", "pair": "k_leja_pair"}.get(form)
+    path = os.path.join(ROOT, "profiles", f"{name}_{precision}_channels3d_{round(n_cells ** (1 / 3))}.md")
     try:
-        sha = kernel_sources_sha()
+        sha = kernel_sources_sha(form)
         vals = {}
         for line in open(path):
             if ":" in line and line.startswith("- "):
@@ -231,7 +281,7 @@ def recorded_traffic(precision: str, n_cells: int):
                 vals[k.strip()] = v.strip()
         if vals.get("kernel sources sha256[:16]") != sha:
             return None
-        return float(vals["dram bytes per cell-term"]) * n_cells
+        return float(vals["dram bytes per cell-term" if form == "single" else "dram bytes per cell-pair"]) * n_cells
     except (OSError, KeyError, ValueError):
         return None
 
@@ -604,14 +654,19 @@ def main(args):
     ms, value = aggregate(r32["ms"], N, K, world, dev)
     peak, peak_kind = measured_peaks()
     b32 = leja_term_bytes("fp32_bulk", r32["leja_coefs"])
-    # a Leja term moves the coefficients once and q in and out; the odd terms
-    # also read and write P: 48 B per cell for odd m, 32 B for even m with the
-    # couplings-only copy (52 and 36 with the diagonal)
-    sec_leja = r32["t_terms_ms"] / 1e3
-    bpc = term_bytes_per_cell(b32, [m for s in r32["degrees"] for m in s[1:]], r32["lagged"])
-    achieved = bpc * N / sec_leja / 1e9 if r32["n_terms"] else None
-    effective = b32 * N * r32["n_terms"] / sec_leja / 1e9 if r32["n_terms"] else None
-    traffic = recorded_traffic("fp32_bulk", N)
+    deg32 = [m for s in r32["degrees"] for m in s[1:]]
+    form = term_form(r32["n_leja"], r32["n_terms"])
+    source = f"{peak_kind} hbm_gbs (MEASURED_PEAKS.json)" if peak_kind == "measured" else "fallback 6.8 TB/s"
+    roof = leja_roofline(form, "float", 3, b32, deg32, r32["lagged"], N, r32["t_terms_ms"], r32["n_terms"],
+                         r32["n_leja"], peak, source)
+    bpc = leja_bytes(form, b32, deg32, r32["lagged"])
+    per_launch = 2 if form == "pair" else 1   # terms
+    if bpc:
+        roof["algorithmic_bytes_per_cell_per_launch"] = per_launch * bpc / max(r32["n_terms"], 1)
+    roof["launch_ms_avg"] = per_launch * roof["term_ms_avg"]
+    roof["timing"] = ("CUDA events on the launching stream around each chunk of term launches (gaps and "
+                      "launches after the stop included: the per-term time is an upper bound)")
+    roof["traffic"] = recorded_traffic(form, "fp32_bulk", N)
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": K, "warmup": Wu,
         "ms_per_step": ms / K, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -626,31 +681,20 @@ def main(args):
         "gpu_launches": r32["launches"],
         "leja": {"degrees_per_step": [s[1:] if s[0] == 1 else s for s in r32["degrees"]],
                  "terms_timed": r32["n_terms"], "alpha": r32["alpha"], "beta": r32["beta"]},
-        "roofline": {"kernel": "k_leja_term<float,4,3>",
-                     "bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                     "frac": achieved / peak if achieved else None, "traffic": traffic,
-                     "peak_source": f"{peak_kind} hbm_gbs (MEASURED_PEAKS.json)" if peak_kind == "measured"
-                     else "fallback 6.8 TB/s",
-                     "algorithmic_bytes_per_cell_per_launch": bpc / max(r32["n_terms"], 1),
-                     "algorithmic_bytes_per_cell": {"odd_terms": b32, "even_terms": b32 - P_BYTES},
-                     "launch_ms_avg": r32["t_terms_ms"] / max(r32["n_terms"], 1),
-                     "timing": "CUDA events on the launching stream around each chunk of term "
-                               "launches (gaps and launches after the stop included: the "
-                               "per-term time is an upper bound)",
-                     "effective_gbs_at_odd_term_bytes": effective,
-                     "term_ms_avg": r32["t_terms_ms"] / max(r32["n_terms"], 1)},
+        "roofline": roof,
         "setup": r32["info"],
     }
     if not args.no_fp64:
         r64 = run_gpu(E, torch, wl, "fp64", K, Wu, dev, world, capture_first=check)
         ms64, value64 = aggregate(r64["ms"], N, K, world, dev)
         b64 = leja_term_bytes("fp64", r64["leja_coefs"])
-        bpc64 = term_bytes_per_cell(b64, [m for s in r64["degrees"] for m in s[1:]], r64["lagged"])
-        ach64 = bpc64 * N / (r64["t_terms_ms"] / 1e3) / 1e9 if r64["n_terms"] else None
+        bpc64 = leja_bytes(term_form(r64["n_leja"], r64["n_terms"]), b64,
+                           [m for s in r64["degrees"] for m in s[1:]], r64["lagged"])
+        ach64 = bpc64 * N / (r64["t_terms_ms"] / 1e3) / 1e9 if bpc64 and r64["n_terms"] else None
         rel = float(np.linalg.norm(r32["T"] - r64["T"]) / np.linalg.norm(r64["T"]))
         line["fp64"] = {"value": value64, "ms_per_step": ms64 / K,
                         "achieved_gbs": ach64,
-                        "algorithmic_bytes_per_cell_per_launch": bpc64 / max(r64["n_terms"], 1),
+                        "algorithmic_bytes_per_cell_per_term": bpc64 / max(r64["n_terms"], 1) if bpc64 else None,
                         "term_ms_avg": r64["t_terms_ms"] / max(r64["n_terms"], 1),
                         "degrees_per_step": [s[1:] if s[0] == 1 else s for s in r64["degrees"]]}
         line["speedup_fp32_bulk_vs_fp64"] = ms64 / ms
@@ -770,7 +814,7 @@ def run_coupled(E, torch, wl, scheme, precision, steps, warmup, dev, capture_fir
     torch.cuda.synchronize()
     e0 = torch.cuda.Event(enable_timing=True)
     e1 = torch.cuda.Event(enable_timing=True)
-    cg_it, lin_it, degrees, launches, t_terms, n_terms, scheds = [], [], [], 0, 0.0, 0, []
+    cg_it, lin_it, degrees, launches, t_terms, n_terms, n_leja, scheds = [], [], [], 0, 0.0, 0, 0, []
     e0.record(stream)
     for _ in range(steps):
         s1, s2 = step()
@@ -781,6 +825,7 @@ def run_coupled(E, torch, wl, scheme, precision, steps, warmup, dev, capture_fir
         launches += s1.launches + s2.launches
         t_terms += s2.t_terms_ms
         n_terms += s2.n_terms_timed
+        n_leja += s2.n_launches_timed
         lagged = bool(s2.terms_lagged)
     e1.record(stream)
     torch.cuda.synchronize()
@@ -789,7 +834,7 @@ def run_coupled(E, torch, wl, scheme, precision, steps, warmup, dev, capture_fir
            "leja_terms_per_step": float(np.mean(degrees)), "launches": launches,
            "leja_coefs": ctx.leja_coefficients, "lagged": lagged,
            "T": T.cpu().numpy(), "rhoc": rc, "t_terms_ms": t_terms, "n_terms": n_terms,
-           "degrees": [m for sc in scheds for m in sc], "first": first}
+           "n_leja": n_leja, "degrees": [m for sc in scheds for m in sc], "first": first}
     if ada["accepted"]:
         out["ros_steps_per_step"] = float(np.mean(ada["accepted"][-steps:]))
         out["ros_rejections_per_step"] = float(np.mean(ada["rejected"][-steps:]))
@@ -844,9 +889,6 @@ def coupled_summary(E, torch, dev, world, K, Wu, check=False):
     h, d, q = runs["erem_fp32_bulk"], runs["erem_fp64"], runs["ros2_fp64"]
     peak, kind = measured_peaks()
     b = leja_term_bytes("fp32_bulk", h["leja_coefs"])  # 2D: the copy's coefficients, q in/out, P in/out
-    h_lag = h["lagged"]
-    bpc = term_bytes_per_cell(b, h["degrees"], h_lag)
-    ach = bpc * wl.n / (h["t_terms_ms"] / 1e3) / 1e9 if h["n_terms"] else None
     rel = lambda a, b_: float(np.linalg.norm(a - b_) / np.linalg.norm(b_))
     out = {
         "workload": "coupled2d_1024", "cells": wl.n, "steps": K, "warmup": Wu, "unit": UNIT,
@@ -860,15 +902,8 @@ def coupled_summary(E, torch, dev, world, K, Wu, check=False):
         "ros2_fp64": {"value": q["value"], "ms_per_step": q["ms"] / K,
                       "stage_iters_per_step": q["stage_iters_per_step"],
                       "rel_l2_vs_erem_fp64": rel(q["T"], d["T"])},
-        "roofline": {"kernel": "k_leja_term<float,4,2>", "bound": "hbm", "achieved": ach, "peak": peak,
-                     "unit": "GB/s", "frac": ach / peak if ach else None, "traffic": None,
-                     "peak_source": f"{kind} hbm_gbs",
-                     "algorithmic_bytes_per_cell": {"odd_terms": b,
-                                                   "even_terms": b if h_lag else b - P_BYTES},
-                     "terms_lagged": h_lag,
-                     "term_ms_avg": h["t_terms_ms"] / max(h["n_terms"], 1),
-                     "note": "the 1024^2 term's working set (about 50 MB) stays in L2, so the "
-                             "achieved rate is not an HBM figure"},
+        "roofline": leja_roofline(term_form(h["n_leja"], h["n_terms"]), "float", 2, b, h["degrees"], h["lagged"],
+                                  wl.n, h["t_terms_ms"], h["n_terms"], h["n_leja"], peak, f"{kind} hbm_gbs"),
     }
     if check and h["first"] is not None:
         out["rel_l2_vs_oracle"] = oracle_coupled_check(
@@ -1078,12 +1113,12 @@ def ensemble_summary(E, torch, dev, world, Wu, members=512, steps=30):
         if prec == "fp32_bulk":
             out.update(summary)
             out["roofline"] = {"kernel": "k_ens_cluster<float,4>", "bound": "hbm",
-                               "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
+                               "achieved": ach, "peak": peak, "unit": "GB/s", "frac": None,
                                "traffic": None, "peak_source": f"{kind} hbm_gbs",
                                "algorithmic_bytes_per_cell_term": b,
-                               "note": "Leja-term bytes only over the whole run; each member's "
-                                       "Leja working set stays in L2 while its cluster runs it, so "
-                                       "the rate can exceed the HBM copy bandwidth"}
+                               "note": "Leja-term bytes only over the whole run; a member's Leja "
+                                       "working set stays in shared memory, or in L2, while its "
+                                       "cluster runs it: no HBM fraction"}
         else:
             out["fp64"] = summary
             out["speedup_fp32_bulk_vs_fp64"] = summary["ms_per_step"] / out["ms_per_step"]
@@ -1137,17 +1172,16 @@ def main_ensemble(args):
                      "substeps_hist": {str(s): r32["substeps"].count(s) for s in sorted(set(r32["substeps"]))},
                      "failed": r32["failed"], "autotune_s": r32["tune_s"], "inputs_s": t_in,
                      "pressure_cg_iters": {"median": float(np.median(cg)), "max": int(max(cg))}},
-        "roofline": {"kernel": "k_ens_cluster<float,4>", "bound": "hbm",
-                     "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
+        "roofline": {"kernel": "k_ens_resident<float,4>, k_ens_cluster<float,4> (by member size)", "bound": "latency",
+                     "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": None,
                      "traffic": None,
                      "peak_source": f"{peak_kind} hbm_gbs (MEASURED_PEAKS.json)" if peak_kind == "measured"
                      else "fallback 6.8 TB/s",
                      "algorithmic_bytes_per_cell_term": b32,
                      "note": "Leja-term bytes only over the whole run (the other passes, about "
                              f"{100 * r32['cell_passes'] / max(r32['cell_terms'], 1):.1f}% of the "
-                             "cell passes, are not counted); each member's Leja working set stays "
-                             "in L2 while its cluster runs it, so the rate can exceed the HBM copy "
-                             "bandwidth"},
+                             "cell passes, are not counted); a member's Leja working set stays in "
+                             "shared memory, or in L2, while its cluster runs it: no HBM fraction"},
     }
     if not args.no_fp64:
         r64 = run_ensemble(E, torch, inputs, "fp64", K, Wu, dev)
@@ -1232,7 +1266,7 @@ def adjoint_runs(E, torch, dev, n, K, Wu, arms):
 
 def adjoint_forward_terms(E, torch, wl, phys, t):
     """The forward run's Leja terms timed on their launching stream: the
-    adjoint workload's dominant kernel (k_leja_term<float,4,3> at 128^3)."""
+    adjoint workload's forward kernel."""
     n = wl.nx
     with E.Context(3, n, n, n, physics=phys, precision="fp32_bulk") as ctx:
         lnk = t(wl.lnk)
@@ -1241,15 +1275,16 @@ def adjoint_forward_terms(E, torch, wl, phys, t):
         T = t(wl.T0)
         ctx.set_state(T, p, lnk, t(wl.phi), t(wl.lam), wl.dt)
         opts = E.leja_opts(tol=wl.tol, time_terms=True)
-        ms, terms, degrees = 0.0, 0, []
+        ms, terms, launches, degrees = 0.0, 0, 0, []
         for _ in range(wl.steps):
             st = ctx.erem_step(T, wl.dt, opts=opts)
             ms += st.t_terms_ms
             terms += st.n_terms_timed
+            launches += st.n_launches_timed
             degrees += list(st.degrees[:st.substeps])
             lagged = bool(st.terms_lagged)
         ncoef = ctx.leja_coefficients
-    return ms, terms, degrees, ncoef, lagged
+    return ms, terms, launches, degrees, ncoef, lagged
 
 
 def adjoint_summary(E, torch, dev, world, n=128, K=2, Wu=1):
@@ -1261,10 +1296,8 @@ def adjoint_summary(E, torch, dev, world, n=128, K=2, Wu=1):
     r, f, q = runs["fp32_bulk"], runs["fp32_bulk_full_tape"], runs["fp64"]
     ms = max_over_ranks(r["ms_per_gradient"], world, dev)
     peak, kind = measured_peaks()
-    tms, terms, degrees, ncoef, lagged = adjoint_forward_terms(E, torch, wl, phys, t)
+    tms, terms, n_leja, degrees, ncoef, lagged = adjoint_forward_terms(E, torch, wl, phys, t)
     b = leja_term_bytes("fp32_bulk", ncoef)
-    h_lag = lagged
-    ach = term_bytes_per_cell(b, degrees, lagged) * wl.n / (tms / 1e3) / 1e9 if terms else None
     rel = lambda a, b_: float(np.linalg.norm(a - b_) / np.linalg.norm(b_))
     return {
         "workload": f"adjoint3d_{n}", "cells": wl.n, "erem_steps": wl.steps, "gradients": K,
@@ -1277,15 +1310,10 @@ def adjoint_summary(E, torch, dev, world, n=128, K=2, Wu=1):
         "rel_l2_gT0_fp32_bulk_vs_fp64": rel(r["gT0"], q["gT0"]),
         "rel_l2_glnk_full_tape_vs_checkpointed": rel(f["glnk"], r["glnk"]),
         "leja_terms_per_forward": r["leja_terms_per_run"],
-        "roofline": {"kernel": "k_leja_term<float,4,3>", "bound": "hbm", "achieved": ach, "peak": peak,
-                     "unit": "GB/s", "frac": ach / peak if ach else None, "traffic": None,
-                     "peak_source": f"{kind} hbm_gbs",
-                     "algorithmic_bytes_per_cell": {"odd_terms": b,
-                                                   "even_terms": b if h_lag else b - P_BYTES},
-                     "terms_lagged": h_lag,
-                     "term_ms_avg": tms / max(terms, 1),
-                     "note": "timed over a 60-step forward run; a 128^3 term moves 109 MB, "
-                             "partly served by the 129 MB L2"},
+        "roofline": dict(leja_roofline(term_form(n_leja, terms), "float", 3, b, degrees, lagged, wl.n, tms, terms,
+                                       n_leja, peak, f"{kind} hbm_gbs"),
+                         note="timed over a 60-step untaped forward run; a 128^3 launch's working set "
+                              "is partly served by the 129 MB L2"),
     }
 
 

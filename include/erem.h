@@ -123,11 +123,13 @@ typedef struct {
   int n_terms_timed;    /* time_terms: Leja terms those chunks computed       */
   int launches;         /* CUDA kernels this call launched                    */
   int n_launches_timed; /* time_terms: Leja kernel launches in t_terms_ms
-                           (those after the stop included)                   */
+                           (those after the stop included); a launch computes
+                           one term, two (large 3D grids, FP32-bulk) or all of
+                           a chunk (grids whose working set fits on the chip) */
   int degree_phi2;      /* erem_step_forced: degree of the phi_2 interpolation */
   int terms_lagged;     /* 1: the Leja terms of this call took each stopping
-                           test in the next launch (small grids, untaped):
-                           the running sum was updated at every term         */
+                           test while a later term ran (small grids): the
+                           running sum was updated at every term             */
 } erem_stats;
 
 typedef struct erem_ctx erem_ctx;

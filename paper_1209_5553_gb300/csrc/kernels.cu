@@ -1900,8 +1900,8 @@ __global__ void k_cg_newdir(const Tz* __restrict__ z, const double* __restrict__
   }
 }
 
-// Ad = A d; (d, Ad) -> alpha.  With k_cg_newdir at 128^3: 10 + 41 us where
-// forming d inside took 91, at 1024^2 6 + 21 instead of 40 (FP64 operations
+// Ad = A d; (d, Ad) -> alpha.  With k_cg_newdir at 128^3: 10 + 38 us where
+// forming d inside took 91, at 1024^2 6 + 19 instead of 40 (FP64 operations
 // per cell in 3D: 1 + 8 instead of 23).
 __global__ void k_cg_dir(PresArr a, const double* __restrict__ d, Geo g, double* part, unsigned* cnt,
                          Ctrl* ctrl) {
