@@ -2497,9 +2497,9 @@ k_mg_coarse_apply(const float* __restrict__ inv, const float* __restrict__ b, fl
 // is on the way down), takes the right-hand side from CTA 0's shared memory and
 // writes its part of the correction back.  The first sweep from zero and the
 // prolongation are formed where the next sweep reads them.  Every value has the
-// bits of the single launches.  Pressure at 128^3: 25 us, where the product with
+// bits of the single launches.  Pressure at 128^3: 24 us, where the product with
 // the coarsest inverse alone took 37.6; stage systems at 512^2 (64^2, 32^2 and
-// 16^2, one CTA): 19.6 us, half of it in loading the operators and in the 40
+// 16^2, one CTA): 19.4 us, about half of it in loading the operators and in the 40
 // sweeps of the coarsest level.
 // ---------------------------------------------------------------------------
 constexpr int kSmallThreads = 1024;
@@ -3152,7 +3152,7 @@ __global__ void k_smg_jacobi(MgN L, const float* __restrict__ rhs, const float* 
 // where the second reads it).  These levels are launch-bound (1.7 us a sweep at
 // 512^2 and below): four launches of a level in place of six, and the same
 // values and order of sums as sweep by sweep.  A V-cycle at 512^2, with the small
-// levels in k_smg_small: 59 -> 46 us.
+// levels in k_smg_small: 59 -> 45 us.
 __global__ void k_smg_jacobi2(MgN L, const float* __restrict__ rhs, float* __restrict__ xo, float w) {
   auto first = [&](int j, int, int, int) { return w * L.Dinv[j] * rhs[j]; };
   for (int i = blockIdx.x * NT + threadIdx.x; i < L.g.N; i += gridDim.x * NT) {
@@ -3542,7 +3542,8 @@ int blocks_cells(const erem_ctx* c) { return grid_for(c, c->N); }
 // BiCGSTAB passes: a block's sum takes five FP64 operations per thread, as much
 // as the cells' own where every thread has one, so a thread takes up to four
 // cells while there are two blocks per SM (512^2: the five passes of an
-// iteration 66 -> 42 us, 9 of them from forming beta once)
+// iteration 66 -> 42 us, 9 of them from forming beta once; 37 with the block
+// sums of device_common.cuh)
 int blocks_bicg(const erem_ctx* c) {
   return std::min(grid_for(c, c->N), std::max(2 * c->sm_count, grid_for(c, c->N / 4)));
 }
