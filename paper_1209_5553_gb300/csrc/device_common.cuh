@@ -288,6 +288,31 @@ __device__ __forceinline__ double div_newton(double n, double d) {
   return fma(fma(-d, q, n), y, q);
 }
 
+// Compensated FP32 sum of squares, hi + lo, with the range of FP64: from 2^100 on
+// (by a square or by the sum) it is kept times 2^-64, so that only a square that
+// is itself infinite makes it so.  Newton vectors of converging interpolations
+// reach ||q||^2 of 10^50 and more, and FP32 ends at 3.4e38.  What a scaled sum
+// loses of its small terms (below 2^-62) is beyond FP64's precision of a sum above
+// 2^100.  With sc = 1 every operation has the bits of the plain pair, and the
+// range costs a maximum, a comparison and a branch that is not taken.
+constexpr float kSquareBig = 0x1p100f, kSquareDown = 0x1p-64f;
+struct SquareSum {
+  float hi = 0.f, lo = 0.f, sc = 1.f;
+  __device__ __forceinline__ void down() {
+    if (sc != 1.f) return;
+    sc = kSquareDown;
+    hi *= kSquareDown;
+    lo *= kSquareDown;
+  }
+  __device__ __forceinline__ void add(float sq) {
+    if (fmaxf(hi, sq) > kSquareBig) down();
+    const float s = fmaf(sq, sc, hi);
+    const float bp = s - hi;
+    lo += (hi - (s - bp)) + fmaf(sq, sc, -bp);
+    hi = s;
+  }
+};
+
 // The Leja copy of J is interleaved per warp tile of T = 32 VEC cells: the
 // tile's NC coefficient arrays D W E S N (B T) follow one another, T values
 // each.  A warp whose lanes own 32 consecutive VEC-cell vectors reads each

@@ -587,7 +587,9 @@ __global__ void __launch_bounds__(kEnsThreads, 2) k_ens_cluster(EnsRun R) {
 // passes per step use them).
 //
 // Arithmetic and decisions are those of k_ens_cluster; only the order in which
-// the squares enter ||q_m||^2 differs.
+// the squares enter ||q_m||^2 differs, and in FP32-bulk their sum is a float pair
+// (48 bits) with FP64's range: as there, an estimate is non-finite where the
+// squares of one vector's cells overflow FP32, not where their sum does.
 //
 // What bounds it: on small members the control step of a pass (about 25 FP64
 // operations in sequence, 64 cycles each, and a reduction over the cluster),
@@ -622,7 +624,9 @@ __device__ __forceinline__ void ens_ld_remote(Tq (&r)[VEC], unsigned p) {
   for (int k = 0; k < VEC; ++k) r[k] = d[k];
 }
 
-// Compensated FP32 sums: x += y, and the sum over a warp in every lane.
+// Compensated FP32 sums: x += y, and the sum over a warp in every lane.  A pair
+// that is kept times 2^-64 (SquareSum) carries the sign bit in x: sums of squares
+// are not negative.
 __device__ __forceinline__ void ens_add_pair(float2& x, float2 y) {
   const float s = x.x + y.x;
   const float bp = s - x.x;
@@ -750,7 +754,7 @@ __global__ void __launch_bounds__(kEnsThreads, 1) k_ens_resident(EnsRun R) {
           Tq* qo = qs + (size_t)(d.m & 1) * nvb * VEC;
           const unsigned in_off = (unsigned)((d.m - 1) & 1) * (unsigned)nvb * 16u;
           const bool addP = d.m >= 2;
-          float s_hi = 0.f, s_lo = 0.f;
+          SquareSum ss;
 #pragma unroll
           for (int k = 0; k < kResKV; ++k) {
             const int mk = mask[k];
@@ -812,18 +816,17 @@ __global__ void __launch_bounds__(kEnsThreads, 1) k_ens_resident(EnsRun R) {
               float sq = 0.f;
 #pragma unroll
               for (int i = 0; i < VEC; ++i) sq = fmaf(out[i], out[i], sq);
-              const float s = s_hi + sq;
-              const float bp = s - s_hi;
-              s_lo += (s_hi - (s - bp)) + (sq - bp);
-              s_hi = s;
+              ss.add(sq);
             } else {
 #pragma unroll
               for (int i = 0; i < VEC; ++i) r = fma(out[i], out[i], r);
             }
           }
           if constexpr (sizeof(Tq) == 4) {
-            const float2 w = ens_warp_pair(make_float2(s_hi, s_lo));
-            r = __hiloint2double(__float_as_int(w.x), __float_as_int(w.y));   // the pair's bits
+            const bool down = __any_sync(0xffffffffu, ss.sc != 1.f);
+            if (down) ss.down();
+            const float2 w = ens_warp_pair(make_float2(ss.hi, ss.lo));
+            r = __hiloint2double(__float_as_int(down ? -w.x : w.x), __float_as_int(w.y));   // the pair's bits
           } else {
             r = warp_sum(r);
           }
@@ -906,12 +909,23 @@ __global__ void __launch_bounds__(kEnsThreads, 1) k_ens_resident(EnsRun R) {
               tot = warp_max(a);
             } else if constexpr (sizeof(Tq) == 4) {
               float2 a = make_float2(0.f, 0.f);   // pairs: FP32 operations, four cycles each
+              int neg = 0;
 #pragma unroll
-              for (int u = 0; u < NJ; ++u)
-                ens_add_pair(a, make_float2(__int_as_float(__double2hiint(x[u])),
-                                            __int_as_float(__double2loint(x[u]))));
+              for (int u = 0; u < NJ; ++u) neg |= __double2hiint(x[u]);
+              const bool down = __any_sync(0xffffffffu, neg < 0);
+#pragma unroll
+              for (int u = 0; u < NJ; ++u) {
+                float2 y = make_float2(__int_as_float(__double2hiint(x[u])),
+                                       __int_as_float(__double2loint(x[u])));
+                if (down) {   // all of them times 2^-64
+                  const float sc = __float_as_int(y.x) < 0 ? 1.f : kSquareDown;
+                  y = make_float2(fabsf(y.x) * sc, y.y * sc);
+                }
+                ens_add_pair(a, y);
+              }
               a = ens_warp_pair(a);
               tot = f2d_fast(a.x) + f2d_fast(a.y);
+              if (down) tot *= 0x1p64;
             } else {
               double a = x[0];
 #pragma unroll
