@@ -562,9 +562,12 @@ erem_status leja_interp(erem_ctx* c, const double* u, const double* fused_T, int
       EREM_TRY(prepare_dd(c, S, *M_avail, s, phi));
       if (slot0 && c->tape_used + ((size_t)mcap + 1 + lag) * qbytes > c->tape_cap) {
         // the tape cannot hold the longer interpolation: go on untaped (the
-        // remaining terms continue from the last taped slot)
+        // remaining terms continue from the last taped slots)
         EREM_CUDA(c, cudaMemcpyAsync(c->q[qin], slot0 + (size_t)(end)*qbytes, qbytes,
                                      cudaMemcpyDeviceToDevice, s));
+        if (res)  // ... whose P is two terms behind: the next launch also reads q_{end-1}
+          EREM_CUDA(c, cudaMemcpyAsync(c->q[qin ^ 1], slot0 + (size_t)(end - 1) * qbytes, qbytes,
+                                       cudaMemcpyDeviceToDevice, s));
         slot0 = nullptr;
         c->rec_ok = false;
       }
