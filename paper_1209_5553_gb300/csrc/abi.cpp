@@ -509,7 +509,7 @@ erem_status leja_interp(erem_ctx* c, const double* u, const double* fused_T, int
   while (true) {
     const int last = (forced ? forced : *M_avail) + lag;
     if (pair) chunk += chunk & 1;
-    const int end = std::min(last, m + chunk - 1);
+    const int end = leja_chunk_end(m, chunk, last, forced);
     if (o.time_terms) cudaEventRecord(c->ev[2 * chunks.size()], s);
     if (res) {
       EREM_CUDA(c, launch_leja_res(c, m, end, *M_avail + 1, forced && end == last ? 0 : 1,

@@ -411,6 +411,14 @@ void launch_leja_term_lag(const erem_ctx* c, int m, int qin, double cg, cudaStre
 bool leja_res_fits(erem_ctx* c);
 constexpr int kResLag = 2;        // terms past the table's last one that complete P
 constexpr int kResTerms = 240;    // terms of one launch, at most
+// The last term of the launches that start at term m: `chunk` terms, up to
+// `last`.  A forced interpolation has tape slots for q_0 .. q_forced only, so a
+// launch that keeps its last vectors (any but the last one) ends there at most.
+inline int leja_chunk_end(int m, int chunk, int last, int forced) {
+  const int end = m + chunk - 1;
+  if (end >= last) return last;
+  return forced && m <= forced && end > forced ? forced : end;
+}
 size_t res_msg_bytes(const erem_ctx* c);
 size_t res_part_bytes(const erem_ctx* c);
 cudaError_t launch_leja_res(erem_ctx* c, int m0, int m1, int ndd, int keep_q, int tape_to, char* tape,

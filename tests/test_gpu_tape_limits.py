@@ -104,3 +104,13 @@ def test_full_tape_of_one_long_step(prec):
     assert a[0] == b[0] and a[0][0][1] > 48
     assert a[1] == b[1]
     assert np.array_equal(a[2], b[2]) and np.array_equal(a[3], b[3])
+
+
+@pytest.mark.parametrize("degree", [237, 238, 239, 240, 241, 479, 480])
+def test_forced_degrees_at_the_end_of_a_launch(degree):
+    # a launch takes 240 terms; the arena holds the q_0 .. q_degree of this
+    # step and nothing more (FP32's range ends before such degrees)
+    torch = pytest.importorskip("torch")
+    pr = Problem(torch, "fp64")
+    dt = pr.long_step()
+    same(pr.run(dt, degree + 1, replay=[1, degree]), pr.run(dt, replay=[1, degree]))
