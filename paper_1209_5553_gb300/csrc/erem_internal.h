@@ -419,6 +419,12 @@ inline int leja_chunk_end(int m, int chunk, int last, int forced) {
   if (end >= last) return last;
   return forced && m <= forced && end > forced ? forced : end;
 }
+// The numbers that mark a launch's messages go up from launch to launch and
+// start over long before they wrap.  That clears the messages, so only the first
+// launch of an interpolation does it: one that continues (m0 > 1) still needs the
+// partial sums of the launch before.
+constexpr unsigned kResBaseTop = 1u << 30;
+inline bool res_renumbers(unsigned base, int m0) { return m0 == 1 && base > kResBaseTop; }
 size_t res_msg_bytes(const erem_ctx* c);
 size_t res_part_bytes(const erem_ctx* c);
 cudaError_t launch_leja_res(erem_ctx* c, int m0, int m1, int ndd, int keep_q, int tape_to, char* tape,

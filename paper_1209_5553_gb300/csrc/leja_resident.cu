@@ -625,9 +625,8 @@ cudaError_t launch_leja_res(erem_ctx* c, int m0, int m1, int ndd, int keep_q, in
   a.m0 = m0;
   a.m1 = m1;
   a.keep_q = keep_q;
-  // the numbers of the terms go up from launch to launch (no message of an
-  // earlier one matches); back to zero long before they wrap
-  if (c->res_base > (1u << 30)) {
+  // no message of an earlier launch carries this one's numbers
+  if (res_renumbers(c->res_base, m0)) {
     cudaError_t e = cudaMemsetAsync(c->res_msg, 0, res_msg_bytes(c), s);
     if (e == cudaSuccess)
       e = cudaMemsetAsync(c->res_part, 0, res_part_bytes(c), s);
