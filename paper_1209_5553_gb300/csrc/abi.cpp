@@ -481,8 +481,7 @@ erem_status leja_interp(erem_ctx* c, const double* u, const double* fused_T, int
   }
   char* slot0 = nullptr;
   if (c->rec_ok && phi == 1) {
-    // the resident form also keeps the vectors past the table's last term
-    const size_t need = (size_t)(forced ? forced : *M_avail + (res ? kResLag : 0)) + 1;
+    const size_t need = (size_t)(forced ? forced : *M_avail) + 1;
     if (c->tape_used + need * qbytes <= c->tape_cap) {
       slot0 = c->tape + c->tape_used;
       c->rec.q_off.push_back(c->tape_used);
@@ -513,7 +512,7 @@ erem_status leja_interp(erem_ctx* c, const double* u, const double* fused_T, int
     if (o.time_terms) cudaEventRecord(c->ev[2 * chunks.size()], s);
     if (res) {
       EREM_CUDA(c, launch_leja_res(c, m, end, *M_avail + 1, forced && end == last ? 0 : 1,
-                                   slot0 ? (forced ? forced : end) : 0, slot0, qbytes, cg, s));
+                                   slot0 ? (forced ? forced : *M_avail) : 0, slot0, qbytes, cg, s));
       qin = end & 1;
     }
     for (int mm = m; pair && mm <= end; mm += 2) {
@@ -560,17 +559,22 @@ erem_status leja_interp(erem_ctx* c, const double* u, const double* fused_T, int
     if (end >= *M_avail + lag) {  // table exhausted below m_max: extend it
       *M_avail = mcap;
       EREM_TRY(prepare_dd(c, S, *M_avail, s, phi));
-      if (slot0 && c->tape_used + ((size_t)mcap + 1 + lag) * qbytes > c->tape_cap) {
-        // the tape cannot hold the longer interpolation: go on untaped (the
-        // remaining terms continue from the last taped slots)
-        EREM_CUDA(c, cudaMemcpyAsync(c->q[qin], slot0 + (size_t)(end)*qbytes, qbytes,
-                                     cudaMemcpyDeviceToDevice, s));
-        if (res)  // ... whose P is two terms behind: the next launch also reads q_{end-1}
-          EREM_CUDA(c, cudaMemcpyAsync(c->q[qin ^ 1], slot0 + (size_t)(end - 1) * qbytes, qbytes,
+      const bool fits = slot0 && c->tape_used + ((size_t)mcap + 1) * qbytes <= c->tape_cap;
+      if (slot0 && !fits) {
+        // the tape cannot hold the longer interpolation: go on untaped.  The
+        // remaining terms continue from the last taped slot, or (resident) from
+        // the two vectors past the old table, which are in the buffers
+        if (!res)
+          EREM_CUDA(c, cudaMemcpyAsync(c->q[qin], slot0 + (size_t)(end)*qbytes, qbytes,
                                        cudaMemcpyDeviceToDevice, s));
         slot0 = nullptr;
         c->rec_ok = false;
       }
+      // the longer table has slots for those two (the table of a resident form
+      // ends kResLag terms before the launch does)
+      for (int k = end - kResLag + 1; fits && res && k <= std::min(end, *M_avail); ++k)
+        EREM_CUDA(c, cudaMemcpyAsync(slot0 + (size_t)k * qbytes, c->q[k & 1], qbytes,
+                                     cudaMemcpyDeviceToDevice, s));
     }
     m = end + 1;
     if (!res) chunk = 8;

@@ -62,10 +62,10 @@ constexpr long long kResSpin = 1 << 21;      // polls before a wait gives up (ab
 struct ResArgs {
   const void* jl;      // Leja copy of J (tile-interleaved)
   const void* r0;      // diagonal-free copy: x = 0 row sums
-  char* q;             // tape: q_m at q + m qstride; null: in qb[m & 1]
+  char* q;             // tape: q_m at q + m qstride up to q_{tape_to}, all of them written
   size_t qstride;
-  void* qb[2];
-  int tape_to;         // q_1 .. q_{tape_to} are written to their slots (tape)
+  int tape_to;         // (0 without a tape)
+  void* qb[2];         // other q_m that are kept: qb[m & 1]
   int nxi, ndd;        // entries of the tables
   double* P;
   const double* p0;    // m = 1: P = d_0 p0
@@ -124,7 +124,7 @@ __device__ __forceinline__ bool get_msg(Tq (&r)[VEC], const ulonglong2* p, unsig
 
 template <typename Tq>
 __device__ __forceinline__ Tq* q_of(const ResArgs& a, int m) {
-  return a.q ? (Tq*)(a.q + (size_t)m * a.qstride) : (Tq*)a.qb[m & 1];
+  return a.q && m <= a.tape_to ? (Tq*)(a.q + (size_t)m * a.qstride) : (Tq*)a.qb[m & 1];
 }
 
 template <typename Tq, int VEC>
@@ -592,10 +592,11 @@ bool leja_res_fits(erem_ctx* c) {
   return c->prec == EREM_FP32_BULK || nv <= 384 + c->Np / res_vec(c) / 110;
 }
 
-// Terms m0 .. m1 in one launch (see k_leja_res); q_{m0-1} in the ping-pong
-// buffer of its parity, or in slot m0 - 1 of the tape, which also takes q_m up
-// to tape_to; the last two vectors are written when keep_q is set.  dd_dev
-// holds ndd entries.
+// Terms m0 .. m1 in one launch (see k_leja_res).  With a tape q_m is read from
+// and written to its slot up to tape_to (the slots of an interpolation end with
+// its table or forced degree); past it, and without a tape, the ping-pong buffer
+// of m's parity holds q_{m0-1} and q_{m0-2} and takes the last two vectors when
+// keep_q is set.  dd_dev holds ndd entries.
 cudaError_t launch_leja_res(erem_ctx* c, int m0, int m1, int ndd, int keep_q, int tape_to, char* tape,
                             size_t qbytes, double cg, cudaStream_t s) {
   const int rows = c->res_hy * c->res_hz;
