@@ -312,6 +312,16 @@ struct SquareSum {
     hi = s;
   }
 };
+// The same for a thread that adds at most 1 / sc squares: all of them times sc, a
+// power of two, so that the sum stays in range as long as each square does, with
+// no test and no further register.  The bits are those of the plain pair unless a
+// square is below 2^-126 / sc.
+__device__ __forceinline__ void add_square(float sq, float sc, float& hi, float& lo) {
+  const float s = fmaf(sq, sc, hi);
+  const float bp = s - hi;
+  lo += (hi - (s - bp)) + fmaf(sq, sc, -bp);
+  hi = s;
+}
 
 // The Leja copy of J is interleaved per warp tile of T = 32 VEC cells: the
 // tile's NC coefficient arrays D W E S N (B T) follow one another, T values

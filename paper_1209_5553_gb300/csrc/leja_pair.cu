@@ -56,6 +56,7 @@ struct PairArgs {
   int m, m_end;        // terms m and m + 1; tests up to term m_end
   int px, ny, nz, rows, zc, nby;   // block: rows x zc planes; blocks in y
   int cf_bytes, q0_bytes, q1_bytes, p_bytes;   // shared memory of one plane of each
+  float sq_scale;      // 2^-k, at least as many squares as a thread adds up to (planes)
   double* part;
   unsigned* cnt;
   Ctrl* ctrl;
@@ -172,15 +173,12 @@ __device__ __forceinline__ void pair_stencil(float (&out)[4], const float (&c)[N
   }
 }
 
-// compensated sum of a vector's squares
-__device__ __forceinline__ void add_squares(const float (&a)[4], float& hi, float& lo) {
+// a vector's squares, times sc
+__device__ __forceinline__ void add_squares(const float (&a)[4], float sc, float& hi, float& lo) {
   float sq = 0.0f;
 #pragma unroll
   for (int k = 0; k < 4; ++k) sq = fmaf(a[k], a[k], sq);
-  const float s = hi + sq;
-  const float bp = s - hi;
-  lo += (hi - (s - bp)) + (sq - bp);
-  hi = s;
+  add_square(sq, sc, hi, lo);
 }
 
 template <bool ND, bool FIRST>
@@ -376,7 +374,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_leja_pair(const PairArgs a)
           for (int j = 0; j < 4; ++j) p[j] = fma(dm, w1[j], fma(dm1, w0[j], p[j]));
         }
         stP<4>(a.P + z * plane + cell, p);
-        add_squares(out, h1, l1);
+        add_squares(out, a.sq_scale, h1, l1);
       }
     }
     if (k > 0 && !late && !mbar_wait(bar0 + 16 + 8 * ((k - 1) & 1), ((k - 1) >> 1) & 1)) late = true;
@@ -394,7 +392,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_leja_pair(const PairArgs a)
       const float ql = has_w ? lds1(c1 - 4) : 0.f, qr = has_e ? lds1(c1 + 16) : 0.f;
       pair_stencil<ND>(out, cp, qc, ql, qr, qs, qn, qb, qt, rp, sh2);
       stv<float, 4>(a.qo + zb * plane + cell, out);
-      add_squares(out, h2, l2);
+      add_squares(out, a.sq_scale, h2, l2);
     }
 #pragma unroll
     for (int j = 0; j < NC; ++j)
@@ -434,8 +432,9 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_leja_pair(const PairArgs a)
       S2 = warp_sum(S2);
       if (lane == 0) {
         *a.cnt = 0;
-        stop_test(a.ctrl, m, dm, S1);
-        if (!a.ctrl->done && m + 1 <= a.m_end) stop_test(a.ctrl, m + 1, a.dd[m + 1], S2);
+        const double back = 1.0 / (double)a.sq_scale;   // a power of two
+        stop_test(a.ctrl, m, dm, S1 * back);
+        if (!a.ctrl->done && m + 1 <= a.m_end) stop_test(a.ctrl, m + 1, a.dd[m + 1], S2 * back);
       }
     }
   }
@@ -518,6 +517,8 @@ cudaError_t launch_leja_pair(const erem_ctx* c, int m, int m_end, int qin, doubl
   a.q0_bytes = sh.q0;
   a.q1_bytes = sh.q1;
   a.p_bytes = sh.pl;
+  a.sq_scale = 1.f;
+  while (a.sq_scale * (float)sh.zc > 1.f) a.sq_scale *= 0.5f;
   a.part = c->red_part;
   a.cnt = c->red_cnt;
   a.ctrl = c->ctrl;

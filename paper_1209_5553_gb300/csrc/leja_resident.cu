@@ -155,9 +155,10 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leja_res(const ResArgs a) {
   constexpr int NC = ND ? NCF - 1 : NCF;         // stored ones
   constexpr bool DREG = sizeof(Tq) == 8;         // FP64: the diagonal in registers, more rows fit
   constexpr int NCS = DREG ? NC - 1 : NC;        // coefficients in shared memory
+  constexpr float kSq = 1.f / KV;                // of a thread's squares (add_square)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   // squares per thread, by the parity of the term: a double, or the float pair
-  // of the compensated FP32 sum
+  // of the compensated FP32 sum, times kSq
   __shared__ double s_red[2][kResWork];
   // shifts c/gamma + xi_m, divided differences d_m and |delta d_m| / (scale sqrt(N))
   // from m = m0 - 2 on
@@ -280,6 +281,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leja_res(const ResArgs a) {
   auto publish_norm = [&](int mt) {
     double v;
     if constexpr (sizeof(Tq) == 4) {
+      // the low parts, at most 2^-22 of their pairs, are summed in FP32 (2^-42 of
+      // the sum)
       const float2* r = reinterpret_cast<const float2*>(s_red[mt & 1]) + lane;
       v = f2d_fast(r[0].x);
       float lo = r[0].y;
@@ -287,7 +290,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leja_res(const ResArgs a) {
         v += f2d_fast(r[k * 32].x);
         lo += r[k * 32].y;
       }
-      v += f2d_fast(lo);
+      v = (v + f2d_fast(lo)) * (double)(1.f / kSq);
     } else {
       const double* r = s_red[mt & 1] + lane;
       v = r[0];
@@ -399,12 +402,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leja_res(const ResArgs a) {
           else acc = fma(out[j], out[j], acc);
           qc[k][j] = out[j];
         }
-        if constexpr (sizeof(Tq) == 4) {
-          const float s = s_hi + sq;
-          const float bp = s - s_hi;
-          s_lo += (s_hi - (s - bp)) + (sq - bp);
-          s_hi = s;
-        }
+        if constexpr (sizeof(Tq) == 4) add_square(sq, kSq, s_hi, s_lo);
       }
       if constexpr (sizeof(Tq) == 4) reinterpret_cast<float2*>(s_red[m & 1])[tid] = make_float2(s_hi, s_lo);
       else s_red[m & 1][tid] = acc;
