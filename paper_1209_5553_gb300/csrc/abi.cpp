@@ -1382,6 +1382,8 @@ erem_status erem_create(const erem_grid* grid, const erem_physics* phys, erem_pr
     c->pair_ok = c->smem_optin > 0 && std::atoi(e) != 0;
     if (c->pair_ok) c->res_ok = false;
   }
+  if (const char* e = std::getenv("EREM_WAIT_POLLS"))  // override (0: every wait of the two kernels runs out)
+    c->wait_polls = std::max(0, std::atoi(e));
   c->term_lag = Np <= kLagCells;
   if (const char* e = std::getenv("EREM_TERM_LAG")) c->term_lag = std::atoi(e) != 0;  // override
   const size_t np = (size_t)Np, nf = (size_t)g.ny * g.nz;

@@ -201,6 +201,7 @@ struct erem_ctx {
   // CTAs (allocated on first use), and the number its next launch counts from
   bool res_ok = false;
   bool pair_ok = false;   // two terms per pass on large 3D grids (leja_pair.cu)
+  int wait_polls = -1;    // polls of a wait of these kernels before it gives up (-1: their own limits)
   int smem_optin = 0;             // shared memory a CTA may have
   int res_hy = 0, res_hz = 0;     // rows of a CTA's block (0: not chosen yet)
   void* res_msg = nullptr;

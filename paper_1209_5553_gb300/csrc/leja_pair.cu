@@ -41,7 +41,8 @@ namespace {
 
 constexpr int kPairThreads = 608;    // at most: 576 vectors of a plane and the copying warp
 constexpr int kPairAhead = 2;        // planes fetched into L2 before their copies
-constexpr int kPairSpin = 1 << 22;   // polls of a copy's barrier before giving up
+constexpr int kPairPolls = 1 << 18;   // polls of a barrier before a wait gives up (about a second: a poll in
+                                     // vain took 3.8 us)
 
 struct PairArgs {
   const float* qi;     // q_{m-1}
@@ -57,6 +58,7 @@ struct PairArgs {
   int px, ny, nz, rows, zc, nby;   // block: rows x zc planes; blocks in y
   int cf_bytes, q0_bytes, q1_bytes, p_bytes;   // shared memory of one plane of each
   float sq_scale;      // 2^-k, at least as many squares as a thread adds up to (planes)
+  int polls;           // of a wait for a step's copies or vectors before it gives up
   double* part;
   unsigned* cnt;
   Ctrl* ctrl;
@@ -84,8 +86,8 @@ __device__ __forceinline__ void bulk_prefetch(const void* src, unsigned bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
 }
 // Wait (bounded) for the phase of the given parity; false when the limit ran out.
-__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
-  for (int k = 0; k < kPairSpin; ++k) {
+__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, int polls) {
+  for (int k = 0; k < polls; ++k) {
     unsigned ok;
     asm volatile(
         "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
@@ -276,7 +278,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_leja_pair(const PairArgs a)
   if (copier)
     for (int d = 2; d < 2 + kPairAhead; ++d) ahead(zf + d);
   if (*(volatile int*)&a.ctrl->done) {
-    if (!mbar_wait(bar0, 0) || (K > 1 && !mbar_wait(bar0 + 8, 0)))
+    if (!mbar_wait(bar0, 0, kPairPolls) || (K > 1 && !mbar_wait(bar0 + 8, 0, kPairPolls)))
       atomicOr(&a.ctrl->flags, FLAG_TIMEOUT);
     return;
   }
@@ -307,19 +309,30 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_leja_pair(const PairArgs a)
 
   if (copy_warp) {
     // once q_m is formed on plane z, the couplings' buffer of this step and
-    // plane z - 1 of q_{m-1} are free for the copies of the step after the next
-    if (copier)
+    // plane z - 1 of q_{m-1} are free for the copies of the step after the next.
+    // (The step's own copies have landed then, unless a wait for them ran out: its
+    // barrier may only be announced again when they have.)
+    if (copier) {
+      int issued = min(K, 2);   // steps whose copies were started
       for (int k = 0; k + 2 < K; ++k) {
-        if (!late && !mbar_wait(bar0 + 16 + 8 * (k & 1), (k >> 1) & 1)) late = true;
         const int z = zf + k;
-        const unsigned bar = bar0 + 8 * (k & 1);
+        const unsigned bar = bar0 + 8 * (k & 1), phase = (k >> 1) & 1;
+        if (!mbar_wait(bar0 + 16 + 8 * (k & 1), phase, a.polls) || !mbar_wait(bar, phase, a.polls)) {
+          late = true;
+          break;
+        }
         const bool more = z + 3 < a.nz;
         mbar_expect(bar, (unsigned)tiles(z + 2) * (128u * NC * 4u) + (more ? q0b : 0u) + p_bytes(z + 2));
         load_cf(z + 2, bar);
         if (more) load_q0(z + 3, bar);
         load_P(z + 2, bar);
         ahead(z + 2 + kPairAhead);
+        issued = k + 3;
       }
+      // the block leaves with no copy in flight, also where waits ran out
+      for (int k = max(issued - 2, 0); k < issued; ++k)
+        if (!mbar_wait(bar0 + 8 * (k & 1), (k >> 1) & 1, kPairPolls)) late = true;
+    }
     __syncwarp();
   }
   for (int k = 0; k <= K && !copy_warp; ++k) {
@@ -329,7 +342,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_leja_pair(const PairArgs a)
     if (k < K) {
       rz = rn;
       if (col0 && k + 1 < K) rn = a.r0[(z + 1) * a.ny + y];
-      if (!late && !mbar_wait(bar0 + 8 * (k & 1), (k >> 1) & 1)) late = true;
+      if (!late && !mbar_wait(bar0 + 8 * (k & 1), (k >> 1) & 1, a.polls)) late = true;
       float qc[4], out[4];
       if (own1) {
         {
@@ -377,7 +390,8 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_leja_pair(const PairArgs a)
         add_squares(out, a.sq_scale, h1, l1);
       }
     }
-    if (k > 0 && !late && !mbar_wait(bar0 + 16 + 8 * ((k - 1) & 1), ((k - 1) >> 1) & 1)) late = true;
+    if (k > 0 && !late && !mbar_wait(bar0 + 16 + 8 * ((k - 1) & 1), ((k - 1) >> 1) & 1, a.polls))
+      late = true;
     const int zb = z - 1;   // q_{m+1}
     if (own2 && zb >= z0 && zb < z1) {
       const unsigned c1 = q10 + (unsigned)(((k + 3) & 3) * a.q1_bytes);
@@ -519,6 +533,7 @@ cudaError_t launch_leja_pair(const erem_ctx* c, int m, int m_end, int qin, doubl
   a.p_bytes = sh.pl;
   a.sq_scale = 1.f;
   while (a.sq_scale * (float)sh.zc > 1.f) a.sq_scale *= 0.5f;
+  a.polls = c->wait_polls >= 0 ? c->wait_polls : kPairPolls;
   a.part = c->red_part;
   a.cnt = c->red_cnt;
   a.ctrl = c->ctrl;

@@ -57,7 +57,7 @@ constexpr int kResMaxKV = 4;                 // vectors per thread, at most
 constexpr int kResRing = 4;                  // partials kept per CTA
 constexpr int kResTab = 256;                 // Leja points and differences staged per launch, at most
 constexpr int kResStatic = 16 * 1024;         // static shared memory, at most
-constexpr long long kResSpin = 1 << 21;      // polls before a wait gives up (about a second)
+constexpr int kResPolls = 1 << 21;           // polls before a wait gives up (about a second)
 
 struct ResArgs {
   const void* jl;      // Leja copy of J (tile-interleaved)
@@ -79,6 +79,7 @@ struct ResArgs {
   unsigned base;       // number that marks term m's messages: base + m
   ulonglong2* msg;     // rows: [parity][vector][2] words pairs
   ulonglong2* part;    // partials: [CTA][kResRing]
+  int polls;           // of a wait for a message before it gives up
   Ctrl* ctrl;
 };
 
@@ -108,18 +109,18 @@ __device__ __forceinline__ void put_msg(ulonglong2* p, const Tq (&r)[VEC], unsig
   st_words(p + 1, u.z, u.w, tag);
 }
 template <typename Tq, int VEC>
-__device__ __forceinline__ bool get_msg(Tq (&r)[VEC], const ulonglong2* p, unsigned tag) {
+__device__ __forceinline__ bool get_msg(Tq (&r)[VEC], const ulonglong2* p, unsigned tag, int polls) {
   ulonglong2 a, b;
-  long long k = 0;
+  int k = 0;
   do {
     a = ld_words(p);
     b = ld_words(p + 1);
-  } while (!(tagged(a, tag) && tagged(b, tag)) && ++k < kResSpin);
+  } while (!(tagged(a, tag) && tagged(b, tag)) && ++k < polls);
   const uint4 u = make_uint4((unsigned)a.x, (unsigned)a.y, (unsigned)b.x, (unsigned)b.y);
   const Tq* d = reinterpret_cast<const Tq*>(&u);
 #pragma unroll
   for (int j = 0; j < VEC; ++j) r[j] = d[j];
-  return k < kResSpin;
+  return k < polls;
 }
 
 template <typename Tq>
@@ -320,7 +321,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leja_res(const ResArgs a) {
       // a neighbour row of another CTA
       auto remote = [&](Tq (&r)[VEC], int v) {
         if (first) ldv_cg<Tq, VEC>(r, q0g + (size_t)v * VEC);
-        else ok &= get_msg<Tq, VEC>(r, mi + 2 * (size_t)v, tag - 1u);
+        else ok &= get_msg<Tq, VEC>(r, mi + 2 * (size_t)v, tag - 1u, a.polls);
       };
       float s_hi = 0.f, s_lo = 0.f;
       double acc = 0.0;
@@ -434,8 +435,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leja_res(const ResArgs a) {
         for (int j = 0; j < NB; ++j)
           if (lane + 32 * j < (int)gridDim.x) {
             if (mt >= a.m0)
-              for (long long k = 0; !tagged(w[j], tag); w[j] = ld_words(pp + (size_t)(lane + 32 * j) * kResRing))
-                if (++k >= kResSpin) {
+              for (int k = 0; !tagged(w[j], tag); w[j] = ld_words(pp + (size_t)(lane + 32 * j) * kResRing))
+                if (++k >= a.polls) {
                   ok = false;
                   break;
                 }
@@ -636,6 +637,7 @@ cudaError_t launch_leja_res(erem_ctx* c, int m0, int m1, int ndd, int keep_q, in
   c->res_base += (unsigned)m1 + 1u;
   a.msg = (ulonglong2*)c->res_msg;
   a.part = (ulonglong2*)c->res_part;
+  a.polls = c->wait_polls >= 0 ? c->wait_polls : kResPolls;
   a.ctrl = c->ctrl;
   const void* kern = res_kernel_of(c, kv);
   const size_t smem = res_smem(c, rows);
