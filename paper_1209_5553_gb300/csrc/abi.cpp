@@ -119,7 +119,7 @@ erem_status check_flags(erem_ctx* c) {
   if (c->ctrl_h->flags & FLAG_BAD_INPUT)
     return fail(c, EREM_EINVAL, "negative conductivity, porosity outside [0,1] or non-positive capacity");
   if (c->ctrl_h->flags & FLAG_TIMEOUT)
-    return fail(c, EREM_ETIMEOUT, "a wait of the resident Leja kernel ran out");
+    return fail(c, EREM_ETIMEOUT, "a wait of a Leja kernel ran out");
   return EREM_OK;
 }
 

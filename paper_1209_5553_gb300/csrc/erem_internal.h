@@ -23,7 +23,7 @@ constexpr int kRedSlots = 4;       // reduction values per block
 constexpr double kRowSumNoDiag = 0x1p-28;  // largest relative interior row sum for a diagonal-free Leja copy
 
 // Bits of Ctrl::flags raised by the set-up kernels (and FLAG_TIMEOUT by a wait
-// of the resident Leja kernel that ran out).
+// that ran out in a Leja kernel, the resident one or the one of pairs).
 enum : int { FLAG_NONFINITE = 1, FLAG_BAD_INPUT = 2, FLAG_TIMEOUT = 4 };
 
 // Parameters of the Leja stopping test of one substep (§4.2).
@@ -53,7 +53,7 @@ struct Ctrl {
   int fail;        // m_max reached without passing
   int nonfinite;   // non-finite estimate met
   int m_last;      // last term evaluated
-  int flags;       // FLAG_* from the set-up kernels
+  int flags;       // FLAG_*
   int lin_done;    // linear solver converged (or broke down)
   int lin_it;      // linear solver iterations
   int lin_break;   // linear solver breakdown

@@ -46,3 +46,19 @@ def test_a_wait_that_runs_out_is_an_error(monkeypatch, shape, prec):
     assert err == [E.EREM_ETIMEOUT] * 2 and torch.equal(T, T0)
     again, none = step(None)
     assert not none and torch.equal(again, ref)
+
+
+@pytest.mark.parametrize("shape, prec", [((2, 64, 64, 1), "fp64"), ((3, 96, 128, 128), "fp32_bulk")], ids=str)
+def test_the_message_names_no_other_kernel(monkeypatch, shape, prec):
+    torch = pytest.importorskip("torch")
+    dim, nx, ny, nz = shape
+    n = nx * ny * nz
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to("cuda:0")
+    x = np.tile((np.arange(nx) + 0.5) / nx, ny * nz)
+    monkeypatch.setenv("EREM_WAIT_POLLS", "0")
+    with E.Context(dim, nx, ny, nz, physics=E.Physics(50.0, 40.0, 1.0, 0.0, 80.0, 0), precision=prec) as ctx:
+        T = t(20.0 + 15.0 * x)
+        ctx.set_state(T, t(1.0 - x), t(np.zeros(n)), t(np.full(n, 0.2)), t(np.ones(n)), 0.002)
+        with pytest.raises(E.EremError, match="wait") as err:
+            ctx.erem_step(T, 0.002)
+    assert "resident" not in str(err.value)
