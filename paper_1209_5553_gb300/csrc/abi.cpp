@@ -511,8 +511,18 @@ erem_status leja_interp(erem_ctx* c, const double* u, const double* fused_T, int
     const int end = leja_chunk_end(m, chunk, last, forced);
     if (o.time_terms) cudaEventRecord(c->ev[2 * chunks.size()], s);
     if (res) {
-      EREM_CUDA(c, launch_leja_res(c, m, end, *M_avail + 1, forced && end == last ? 0 : 1,
-                                   slot0 ? (forced ? forced : *M_avail) : 0, slot0, qbytes, cg, s));
+      const cudaError_t e = launch_leja_res(c, m, end, *M_avail + 1, forced && end == last ? 0 : 1,
+                                            slot0 ? (forced ? forced : *M_avail) : 0, slot0, qbytes, cg, s);
+      if (e == cudaErrorCooperativeLaunchTooLarge && m == 1) {
+        // fewer SMs than the device has (a partitioned context): this context's
+        // terms take one launch each from here on
+        cudaGetLastError();
+        c->res_ok = false;
+        if (slot0) c->rec.q_off.pop_back();
+        return leja_interp(c, u, fused_T, S, phi, M_avail, mcap, sp, forced, o, tt, degree, failed, nonfinite, s,
+                           fix);
+      }
+      EREM_CUDA(c, e);
       qin = end & 1;
     }
     for (int mm = m; pair && mm <= end; mm += 2) {
@@ -1377,6 +1387,9 @@ erem_status erem_create(const erem_grid* grid, const erem_physics* phys, erem_pr
     coop = 0;
   }
   c->res_ok = coop != 0 && !std::getenv("EREM_TERM_LAG");
+  c->res_sms = std::min(c->sm_count, kResSms);
+  if (const char* e = std::getenv("EREM_RES_SMS"))  // override: the SMs it is planned for
+    c->res_sms = std::max(1, std::min(std::atoi(e), kResSms));
   c->pair_ok = c->smem_optin > 0 && !std::getenv("EREM_TERM_LAG");
   if (const char* e = std::getenv("EREM_TERM_PAIR")) {  // tuning override: pairs, also on grids that fit on the chip
     c->pair_ok = c->smem_optin > 0 && std::atoi(e) != 0;

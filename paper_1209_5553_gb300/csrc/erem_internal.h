@@ -199,7 +199,8 @@ struct erem_ctx {
   mutable bool last_lag = false;  // the current call ran lagged terms
   // resident Leja kernel (leja_resident.cu): messages and partial sums of its
   // CTAs (allocated on first use), and the number its next launch counts from
-  bool res_ok = false;
+  bool res_ok = false;    // false after a launch the device refused
+  int res_sms = 0;        // SMs it is planned for, one CTA each
   bool pair_ok = false;   // two terms per pass on large 3D grids (leja_pair.cu)
   int wait_polls = -1;    // polls of a wait of these kernels before it gives up (-1: their own limits)
   int smem_optin = 0;             // shared memory a CTA may have
@@ -410,6 +411,7 @@ void launch_leja_term_lag(const erem_ctx* c, int m, int qin, double cg, cudaStre
 // Resident form (leja_resident.cu): terms m0 .. m1 in one cooperative launch,
 // where the grid's Leja working set fits on the chip.
 bool leja_res_fits(erem_ctx* c);
+constexpr int kResSms = 160;      // CTAs of a launch, at most
 constexpr int kResLag = 2;        // terms past the table's last one that complete P
 constexpr int kResTerms = 240;    // terms of one launch, at most
 // The last term of the launches that start at term m: `chunk` terms, up to

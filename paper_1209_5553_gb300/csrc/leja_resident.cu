@@ -52,7 +52,6 @@ namespace {
 constexpr int kResThreads = 512;             // 14 compute warps, a sum warp and a test warp
 constexpr int kResWork = kResThreads - 64;
 constexpr int kResWarps = kResWork / 32;
-constexpr int kResSms = 160;                 // CTAs of a launch, at most
 constexpr int kResMaxKV = 4;                 // vectors per thread, at most
 constexpr int kResRing = 4;                  // partials kept per CTA
 constexpr int kResTab = 256;                 // Leja points and differences staged per launch, at most
@@ -542,7 +541,7 @@ size_t res_smem(const erem_ctx* c, int rows) {
 // the largest block (the slowest CTA decides a term), then the fewest rows
 // that other blocks read.
 void res_blocks(const erem_ctx* c, int* hy, int* hz) {
-  const int sms = std::min(c->sm_count, kResSms);
+  const int sms = c->res_sms;
   const int vrow = c->px / res_vec(c);
   const long long least = std::max(1, kResMinVecs / vrow);
   long long best = -1;
@@ -569,7 +568,7 @@ size_t res_msg_bytes(const erem_ctx* c) {
   const size_t esz = c->prec == EREM_FP32_BULK ? sizeof(float) : sizeof(double);
   return 4 * esz * (size_t)c->Np;   // two buffers of twice the data
 }
-size_t res_part_bytes(const erem_ctx* c) { return sizeof(ulonglong2) * kResRing * (size_t)c->sm_count; }
+size_t res_part_bytes(const erem_ctx* c) { return sizeof(ulonglong2) * kResRing * (size_t)c->res_sms; }
 
 // Whether the grid takes the resident form: its Leja working set fits on the
 // chip and, in FP64, its rows spread well enough.  A block of whole rows is
@@ -595,7 +594,8 @@ bool leja_res_fits(erem_ctx* c) {
 // and written to its slot up to tape_to (the slots of an interpolation end with
 // its table or forced degree); past it, and without a tape, the ping-pong buffer
 // of m's parity holds q_{m0-1} and q_{m0-2} and takes the last two vectors when
-// keep_q is set.  dd_dev holds ndd entries.
+// keep_q is set.  dd_dev holds ndd entries.  The device refuses a launch whose
+// CTAs cannot all run at once (cudaErrorCooperativeLaunchTooLarge).
 cudaError_t launch_leja_res(erem_ctx* c, int m0, int m1, int ndd, int keep_q, int tape_to, char* tape,
                             size_t qbytes, double cg, cudaStream_t s) {
   const int rows = c->res_hy * c->res_hz;
