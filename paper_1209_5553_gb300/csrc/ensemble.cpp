@@ -33,6 +33,21 @@ struct EnsLaunch {
   }
 };
 
+// How a run's members are split into launches: class k (the smallest cluster a
+// member fits on has 2 << k CTAs; 4: none) of [from, to) share one, and what the
+// split was made for.
+struct EnsPlan {
+  struct Part {
+    int from = 0, to = 0, cs = 0;
+    bool res = false;
+  };
+  bool made = false;
+  int max_clusters = 0;
+  std::vector<int> cls;
+  std::vector<double> rate;   // passes per step of each member
+  std::vector<Part> parts;    // the largest classes first
+};
+
 struct erem_ens {
   int n = 0;
   erem_precision prec = EREM_FP64;
@@ -76,6 +91,8 @@ struct erem_ens {
   EnsRun run_key{};
   std::vector<EnsLaunch> key_launches;
   std::vector<EnsLaunch> launches;   // of the next run
+  EnsPlan plan;
+  bool resident_ok = true;           // false: every member works from L2
   int fit_res[5] = {-1, -1, -1, -1, -1}, fit_l2[5] = {-1, -1, -1, -1, -1};   // clusters of 1 << k CTAs at once
   bool graph_ok = true;             // false after a failed capture: direct launches
 
@@ -281,10 +298,8 @@ int fit_clusters(erem_ens* E, int cs, bool res) {
 }
 
 bool fits_resident(const erem_ens* E, int e, int cs) {
-  if (const char* v = std::getenv("EREM_ENS_RESIDENT"))  // tuning override: 0 keeps every member in L2
-    if (std::atoi(v) == 0) return false;
   const erem_ctx* c = E->ctx[e];
-  return ens_res_fits(E->prec, cs, c->ny, c->px, c->jl_nodiag, c->smem_optin);
+  return E->resident_ok && ens_res_fits(E->prec, cs, c->ny, c->px, c->jl_nodiag, c->smem_optin);
 }
 
 // Passes per step of member e: of its last run, else the width of its
@@ -334,50 +349,31 @@ double launch_time(erem_ens* E, const std::vector<int>& who, int cs, bool res) {
   return res ? end : std::max(end, cells / (E->prec == EREM_FP32_BULK ? 110e3 : 41e3));
 }
 
-// The launches of the next run and its queue order.  A given (or tuned)
-// cluster size takes one launch for the members that fit on such a cluster's
-// shared memory and one for the rest.  Otherwise the members are split by the
-// smallest cluster they fit on, neighbouring classes share a launch, and each
-// launch takes the form (shared memory or L2) and the cluster size by which the
-// whole run is shortest.
-erem_status plan_run(erem_ens* E) {
-  const int fixed = E->cfg.cluster_ctas ? E->cfg.cluster_ctas : E->tuned_cs;
-  E->launches.clear();
-  std::vector<std::pair<double, int>> w(E->n);
-  for (int e = 0; e < E->n; ++e) w[e] = {member_weight(E, e), e};
-  std::stable_sort(w.begin(), w.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
-  int pos = 0;
-  auto add = [&](bool res, int cs, const std::vector<char>& in) -> erem_status {
-    EnsLaunch L;
-    L.res = res;
-    L.cs = cs;
-    L.first = pos;
-    for (const auto& x : w)
-      if (in[x.second]) E->order_h[pos++] = x.second;
-    L.count = pos - L.first;
-    if (L.count == 0) return EREM_OK;
-    const int fit = fit_clusters(E, cs, res);
-    if (fit < 1)
-      return efail(E, EREM_ECUDA, "a cluster of " + std::to_string(cs) + " CTAs does not fit the device");
-    L.clusters = std::min(fit, L.count);
-    E->launches.push_back(L);
-    return EREM_OK;
-  };
-  std::vector<char> in(E->n, 0), rest(E->n, 0);
-  if (fixed) {
-    const bool any = fit_clusters(E, fixed, true) > 0;
-    for (int e = 0; e < E->n; ++e) {
-      in[e] = any && fits_resident(E, e, fixed);
-      rest[e] = !in[e];
-    }
-    ENS_TRY(add(true, fixed, in));
-    return add(false, fixed, rest);
+// Whether the plan was made for members like these: the same classes and limit,
+// and no member's passes per step off by more than a quarter (the plan has to
+// promise a fifth before it is taken at all).  Playing the queues of all
+// candidates takes about 1.5 us per member (0.75 ms for 512, as long as a short
+// run's own work); this and the queue order take 0.05 ms.
+bool plan_holds(const erem_ens* E, const std::vector<int>& cls) {
+  const EnsPlan& p = E->plan;
+  if (!p.made || p.max_clusters != E->cfg.max_clusters || p.cls != cls) return false;
+  for (int e = 0; e < E->n; ++e) {
+    const double r = member_rate(E, e);
+    if (!(r <= 1.25 * p.rate[e] && p.rate[e] <= 1.25 * r)) return false;
   }
-  // class k: the smallest cluster of 2 << k CTAs the member fits on
-  std::vector<int> cls(E->n, 4);
-  for (int e = 0; e < E->n; ++e)
-    for (int k = 3; k >= 0; --k)
-      if (fit_clusters(E, 2 << k, true) > 0 && fits_resident(E, e, 2 << k)) cls[e] = k;
+  return true;
+}
+
+// Neighbouring classes share a launch, and each launch takes the form (shared
+// memory or L2) and the cluster size by which the whole run is shortest.
+erem_status make_plan(erem_ens* E, const std::vector<int>& cls) {
+  EnsPlan& p = E->plan;
+  p.made = false;
+  p.max_clusters = E->cfg.max_clusters;
+  p.cls = cls;
+  p.rate.resize(E->n);
+  for (int e = 0; e < E->n; ++e) p.rate[e] = member_rate(E, e);
+  p.parts.clear();
   // best[k]: the shortest time of classes < k, the last launch being [from, k)
   double best[6] = {0.0};
   int from[6] = {0}, size[6] = {0};
@@ -415,8 +411,62 @@ erem_status plan_run(erem_ens* E) {
     resident[5] = false;
   }
   for (int k = 5; k > 0; k = from[k]) {
-    for (int e = 0; e < E->n; ++e) in[e] = cls[e] >= from[k] && cls[e] < k;
-    ENS_TRY(add(resident[k], size[k], in));
+    EnsPlan::Part t;
+    t.from = from[k];
+    t.to = k;
+    t.cs = size[k];
+    t.res = resident[k];
+    p.parts.push_back(t);
+  }
+  p.made = true;
+  return EREM_OK;
+}
+
+// The launches of the next run and its queue order.  A given (or tuned)
+// cluster size takes one launch for the members that fit on such a cluster's
+// shared memory and one for the rest.  Otherwise the members are split by the
+// smallest cluster they fit on, as the plan says.
+erem_status plan_run(erem_ens* E) {
+  const int fixed = E->cfg.cluster_ctas ? E->cfg.cluster_ctas : E->tuned_cs;
+  E->launches.clear();
+  std::vector<std::pair<double, int>> w(E->n);
+  for (int e = 0; e < E->n; ++e) w[e] = {member_weight(E, e), e};
+  std::stable_sort(w.begin(), w.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
+  int pos = 0;
+  auto add = [&](bool res, int cs, const std::vector<char>& in) -> erem_status {
+    EnsLaunch L;
+    L.res = res;
+    L.cs = cs;
+    L.first = pos;
+    for (const auto& x : w)
+      if (in[x.second]) E->order_h[pos++] = x.second;
+    L.count = pos - L.first;
+    if (L.count == 0) return EREM_OK;
+    const int fit = fit_clusters(E, cs, res);
+    if (fit < 1)
+      return efail(E, EREM_ECUDA, "a cluster of " + std::to_string(cs) + " CTAs does not fit the device");
+    L.clusters = std::min(fit, L.count);
+    E->launches.push_back(L);
+    return EREM_OK;
+  };
+  std::vector<char> in(E->n, 0), rest(E->n, 0);
+  if (fixed) {
+    const bool any = fit_clusters(E, fixed, true) > 0;
+    for (int e = 0; e < E->n; ++e) {
+      in[e] = any && fits_resident(E, e, fixed);
+      rest[e] = !in[e];
+    }
+    ENS_TRY(add(true, fixed, in));
+    return add(false, fixed, rest);
+  }
+  std::vector<int> cls(E->n, 4);
+  for (int e = 0; e < E->n; ++e)
+    for (int k = 3; k >= 0; --k)
+      if (fit_clusters(E, 2 << k, true) > 0 && fits_resident(E, e, 2 << k)) cls[e] = k;
+  if (!plan_holds(E, cls)) ENS_TRY(make_plan(E, cls));
+  for (const EnsPlan::Part& p : E->plan.parts) {
+    for (int e = 0; e < E->n; ++e) in[e] = cls[e] >= p.from && cls[e] < p.to;
+    ENS_TRY(add(p.res, p.cs, in));
   }
   return EREM_OK;
 }
@@ -615,6 +665,7 @@ erem_status erem_ensemble_create(int n_members, const erem_grid* grids, const er
   if (cudaMalloc((void**)&E->stage_d, sizeof(double) * maxN) != cudaSuccess) return bail(EREM_ENOMEM);
   if (cudaEventCreate(&E->ev[0]) != cudaSuccess || cudaEventCreate(&E->ev[1]) != cudaSuccess)
     return bail(EREM_ECUDA);
+  if (const char* v = std::getenv("EREM_ENS_RESIDENT")) E->resident_ok = std::atoi(v) != 0;  // tuning override
   if (const char* v = std::getenv("EREM_ENS_GRAPH")) E->graph_ok = std::atoi(v) != 0;  // 0: direct launches
   *out = E;
   return EREM_OK;
