@@ -573,13 +573,15 @@ EREM_API int erem_phi1_divided_differences(int M, const double* xi, double c,
  *
  * On the device every member is a small state machine (G(T^n) -> Leja terms
  * with the stopping test of §4.2 -> substep bookkeeping -> T^{n+1}) whose
- * phases are passes over the member's cells.  One launch runs the whole
- * run: a persistent grid of thread-block clusters takes members from a queue
- * (heaviest first) and each cluster runs its member through every step,
- * with the cluster barrier between passes and the pass's reduction shared
- * through distributed shared memory, so members proceed at their own Leja
- * degrees and substep counts and a member's Leja vectors and coefficients
- * stay in L2 while its cluster works on it.  Stopping, substep doubling and
+ * phases are passes over the member's cells.  A run is up to five launches,
+ * planned by the members' sizes and passes per step: in each a persistent grid
+ * of thread-block clusters takes members from a queue (heaviest first) and
+ * each cluster runs its member through every step, with the cluster barrier
+ * between passes and the pass's reduction shared through distributed shared
+ * memory, so members proceed at their own Leja degrees and substep counts.  A
+ * member's Leja vectors and coefficients stay in its cluster's shared memory
+ * where they fit and the plan finds that faster, else in L2 while its cluster
+ * works on it.  Stopping, substep doubling and
  * the end of the run are decided on the device.  A member is bounded: it
  * stops after steps * (sum over substep levels of 2^l (m_max + 3) + 2) + 2
  * passes at most (EREM_ETIMEOUT).
@@ -595,8 +597,8 @@ typedef enum { EREM_ENS_KEEP_SUBSTEPS = 0, EREM_ENS_RESTART_SUBSTEPS = 1 } erem_
 typedef struct {
   int substep_policy;  /* erem_ens_policy (default KEEP)                    */
   int cluster_ctas;    /* CTAs of the cluster that runs one member: 2, 4, 8
-                          or 16; 0 = 8, or the size erem_ensemble_autotune
-                          chose                                             */
+                          or 16; 0 = planned for each launch, or what
+                          erem_ensemble_autotune chose                      */
   int max_clusters;    /* 0: as many clusters as fit on the device at once */
   int reserved;        /* must be 0                                        */
 } erem_ens_config;
@@ -625,12 +627,12 @@ typedef struct {
   long long cells;       /* sum of the members' cells                      */
   long long cell_terms;  /* sum over members of cells x Leja terms         */
   long long cell_passes; /* sum over members of cells x other passes       */
-  int cluster_ctas;      /* CTAs per cluster of the last run                */
-  int clusters;          /* clusters launched (resident at once)           */
+  int cluster_ctas;      /* CTAs per cluster of the launch with most work  */
+  int clusters;          /* its clusters (resident at once)                */
   int cta_threads;       /* threads per CTA                                */
   int members_failed;
   int graph;             /* 1: the run was replayed from its captured CUDA
-                            graph (uploads, the launch, the read-back);
+                            graph (uploads, launches, the read-back);
                             0: launched directly (capture unavailable)     */
   int reserved;
 } erem_ens_run_stats;
@@ -669,8 +671,8 @@ EREM_API erem_status erem_ensemble_configure(erem_ens* ens, const erem_leja_opts
 
 /* Cluster-size and substep autotuner: runs probe_steps steps of the whole
  * ensemble once to learn every member's substep level and work (the queue
- * order), then once for each cluster size that fits the device (2, 4, 8, 16
- * CTAs), keeps the fastest, and restores every member's temperature
+ * order), then once as planned and once for each cluster size that fits the
+ * device (2, 4, 8, 16 CTAs), keeps the fastest, and restores every member's temperature
  * afterwards.  The timing stands for runs of about probe_steps steps: a
  * short run ends with its heaviest member alone, which favours large
  * clusters, a long one is bound by throughput.  Under the KEEP policy each member then starts at the substep
@@ -678,11 +680,11 @@ EREM_API erem_status erem_ensemble_configure(erem_ens* ens, const erem_leja_opts
  * reach, by doubling).  Errors as erem_ensemble_run. */
 EREM_API erem_status erem_ensemble_autotune(erem_ens* ens, int probe_steps, void* stream);
 
-/* Advance every member by `steps` EREM steps (one kernel launch).  The run
- * (the member states and queue order uploaded from pinned host memory, the
- * persistent launch, the states read back) is captured once as a CUDA graph
- * per run configuration (the members' tables, the options, the cluster
- * shape) and replayed on `stream`; where capture is not available it is
+/* Advance every member by `steps` EREM steps (up to five kernel launches).
+ * The run (the member states and queue order uploaded from pinned host memory,
+ * the persistent launches, the states read back) is captured once as a CUDA
+ * graph per run configuration (the members' tables, the options, the launches)
+ * and replayed on `stream`; where capture is not available it is
  * launched directly (erem_ensemble_run_stats.graph tells which).  Returns
  * when the run is complete.  A member whose Leja interpolation fails (the
  * stopping test not met within m_max terms, or a non-finite estimate: the

@@ -84,7 +84,7 @@ struct erem_ens {
   double* stage_d = nullptr;        // host-pointer staging (largest member)
   cudaEvent_t ev[2] = {nullptr, nullptr};
 
-  // the run as a CUDA graph (state and queue upload, the persistent launch,
+  // the run as a CUDA graph (state and queue upload, the persistent launches,
   // state read-back), captured once per run descriptor and cluster shape
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t run_exec = nullptr;
@@ -531,8 +531,8 @@ void capture_run(erem_ens* E, const EnsRun& R) {
   E->key_launches = E->launches;
 }
 
-// One run: every member advances `steps` steps, one launch of the batched
-// kernel.  A member whose Leja estimate became non-finite (the Newton
+// One run: every member advances `steps` steps, in one launch of a batched
+// kernel for each part of the plan (up to five).  A member whose Leja estimate became non-finite (the Newton
 // vectors or their squares left the range of the Leja precision) or whose
 // interpolation did not meet the test within m_max terms takes the step again
 // at twice the substeps, as erem_step splits a step whose interpolation

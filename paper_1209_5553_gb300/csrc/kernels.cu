@@ -248,7 +248,7 @@ struct JOut {
 
 // FM is the fluid model.  FP64 operations bound this kernel (39 per cell in 3D
 // with the linear fluid; 88 when the upwind choices, extremes and checks were
-// FP64 compares and the row-sum test an FP64 division): 192^3 1070 -> 520 us.
+// FP64 compares and the row-sum test an FP64 division): 192^3 1070 -> 662 us.
 // dX (FM = 1): dX/dT of every cell, written by k_faces.
 template <int FM>
 __global__ void k_cellJ(FaceIn f, const double* __restrict__ dX, JOut o, Geo g, Phys ph,
@@ -2507,9 +2507,9 @@ constexpr int kSmallCtas = 16;
 constexpr int kSmallLevels = 8;
 
 // The cells' coordinates, packed into 16 bits each (a small level has at most
-// 2^12 cells or so; the bits of its three dimensions add up to at most 15): a
-// single SM runs these levels, and two integer divisions per cell and operation
-// would be most of its instructions.
+// 2^12 cells or so; a level whose three dimensions need more than 16 bits is
+// launched by itself): a single SM runs these levels, and two integer divisions
+// per cell and operation would be most of its instructions.
 struct SmallCell {
   const unsigned short* co;
   int bx, by;   // bits of ix and iy
@@ -2803,7 +2803,7 @@ __global__ void k_sumsq(const double* __restrict__ x, Geo g, double* part, unsig
 // = 0: density and viscosity are 1, the means are the pressure couplings
 // themselves, and m is ln K in the caller's layout, read at the x = 0 and x =
 // 1 cells only.  |v| is compared per axis and divided by the face area once
-// per thread (a division per face bounded the pass: 128^3 327 -> 60 us).
+// per thread (a division per face bounded the pass: 128^3 327 -> 116 us).
 template <int FM>
 __global__ void k_pres_post(const double* __restrict__ m, PresArr a, Geo g, Phys ph, double* part,
                             unsigned* cnt, Ctrl* ctrl) {

@@ -24,13 +24,13 @@
 // d_{m-1} q_{m-1} + d_m q_m, as at an odd term of the single form; a substep that
 // stops at m + 1 has P short of d_{m+1} q_{m+1}, which its consumer adds.
 //
-// What bounds it: DRAM moves the 48 bytes and no more (256^3: 792 MB a pair,
-// 5.4 TB/s); a step's instructions (FP64 pipe 42 %, issue 50 %, with 19 warps of
+// What bounds it: DRAM moves the 48 bytes and no more (256^3: 796 MB a pair,
+// 5.7 TB/s); a step's instructions (FP64 pipe 46 %, issue 56 %, with 19 warps of
 // 96 registers) take longer than its copies.  Measured per term, against
-// k_leja_term and k_leja_term_lag: 256^3 74 us (107), 224^3 55 (75), 192^3 38 (48),
-// 128^3 14.6 (17.5), 96 x 400 x 100 24 (26); with the diagonal 224^3 60 (84),
-// 128^3 15.5 (18.2).  With one block barrier per step 256^3 took 82 us, without the
-// fetch into L2 95.
+// k_leja_term and k_leja_term_lag: 256^3 70 us (107), 224^3 53 (75), 192^3 38 (48),
+// 128^3 14.6 (17.3), 96 x 400 x 100 23 (27); with the diagonal 224^3 56 (84),
+// 128^3 16.0 (18.3).  An earlier form took 82 us at 256^3 with one block barrier per
+// step, 95 without the fetch into L2.
 #include <algorithm>
 
 #include "erem_internal.h"
@@ -462,7 +462,7 @@ struct PairShape {
 
 // The block shape: at most one block per SM, the shortest march.  A step takes
 // about 0.9 us + 2.6 ns per vector of its rows (the rows formed for neighbours
-// included), 2.2 us at 256^3, and there are two steps more than planes.
+// included), 2.1 us at 256^3, and there are two steps more than planes.
 PairShape pair_shape(const erem_ctx* c) {
   PairShape best;
   const int nc = c->jl_nodiag ? 6 : 7, vrow = c->px / 4;
@@ -497,8 +497,8 @@ PairShape pair_shape(const erem_ctx* c) {
 
 // Whether the terms run in pairs: FP32-bulk in 3D, at least four rows to a
 // block (fewer, and a block forms half of its rows for its neighbours: rows of
-// up to 384 cells).  At four rows a pair was still 6 % faster than two terms
-// (384 x 160 x 160: 62.7 against 66.5 us a term), at every other size tried from
+// up to 384 cells).  At four rows a pair was still 8 % faster than two terms
+// (384 x 160 x 160: 60.4 against 65.9 us a term), at every other size tried from
 // 1.5 million cells up (smaller grids are resident) 5 to 35 %.  FP64 terms are
 // bound by the FP64 pipe, which rows formed twice would load more.
 bool leja_pair_fits(const erem_ctx* c) {
